@@ -225,6 +225,9 @@ __global__ void __launch_bounds__(RT_THREADS, 2)
             shift(ca, ea, ba);
             shift(cb, eb, bb);
         }
+        // step i0 ends by bringing plane i0 + 5 into plane i0 - 1's slot, which the reads above
+        // use: no warp may get there before every warp has read it
+        __syncthreads();
         float v0 = 0.f, v1 = 0.f, r0 = 0.f, r1 = 0.f;   // the even plane's children of this row
         const int J = (j0 >> 1) + (jj >> 1), K = (k0 >> 1) + pp;
 

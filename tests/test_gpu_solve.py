@@ -334,6 +334,24 @@ def test_batch_equals_alone_and_oracle(ctx):
         assert torch.equal(a, b)
 
 
+def test_batch_of_large_boxes_equals_alone(ctx):
+    """Boxes of 64^3 and up side by side, several replays: the CTAs of different boxes share the
+    SMs, so a kernel whose warps may drift apart (the column-march restriction refilling a plane
+    slot that another warp still reads) shows up as a difference from the box solved alone."""
+    import torch
+    mg = _mg()
+    alpha, s, h = nominal()
+    sides = [64, 128, 96, 64, 128, 96, 64, 128, 64, 96, 128, 64]
+    deltas = [dev(workload.lognormal_delta(n, 1.0, 3000 + b)) for b, n in enumerate(sides)]
+    p = mg.default_params(alpha=alpha, s=s, h=h, tol=1e-8, precision="mixed")
+    alone = [ctx.solve_fifth_force(d, p)[0] for d in deltas]
+    phis = [torch.empty_like(d) for d in deltas]
+    for _ in range(6):
+        ctx.solve_batch(deltas, p, phis=phis)
+        for a, b in zip(phis, alone):
+            assert torch.equal(a, b)
+
+
 def test_batch_mixed_status_per_box(ctx):
     """A box that cannot converge within its cap reports it; the others are unaffected."""
     import torch
