@@ -80,6 +80,10 @@ cudaError_t launch_sweep(const T *in, T *out, const T *f, const double *cptr, in
 {
     if (block < 32 || block > 1024 || block % 32)
         return cudaErrorInvalidValue;
+    if constexpr (sizeof(T) == 8) {
+        if (!B && n >= kSplitMinSweep)
+            return launch_split_sweep(in, out, f, cptr, n, cf, clamp, st);
+    }
     const long long work = (long long)n * n * (n / 2);
     const int g = (int)((work + block - 1) / block);
     if (B) {
@@ -155,6 +159,10 @@ template <typename T>
 cudaError_t launch_residual(const T *phi, const T *f, const double *cptr, int n, CoefT<T> cf, T *r,
                             double2 *partials, int *nblocks, cudaStream_t st, const Fin &fin)
 {
+    if constexpr (sizeof(T) == 8) {
+        if (n >= kSplitMinResid)
+            return launch_split_residual(phi, f, cptr, n, cf, r, partials, nblocks, st, fin);
+    }
     const long long work = (long long)n * n * n;
     const int cap = sizeof(T) == 8 ? kReduceBlocksFp64 : kReduceBlocks;
     const int bs = block_spread(work);
@@ -278,6 +286,8 @@ cudaError_t launch_resid_restrict(const T *v, const T *f, const double *cptr, in
     const long long work = (long long)(n / 2) * (n / 2) * (n / 2);
     const int cap = sizeof(T) == 8 ? kReduceBlocksFp64 : kReduceBlocks;
     if constexpr (sizeof(T) == 8) {
+        if (!B && n >= kSplitMinResid)
+            return launch_split_resid_restrict(v, f, cptr, n, cf, vc, v0c, rc, partials, nblocks, st, fin);
         if (!B && 8 * work <= kChildMaxFine) {   // coarse grids of the FP64 solves
             const long long fine = 8 * work;
             const int bf = block_spread(fine);
@@ -367,6 +377,10 @@ template <typename T>
 cudaError_t launch_coarse_rhs(const T *vc, T *fc, const double *m_fine, double *c_coarse, int nc,
                               CoefT<T> cfc, cudaStream_t st, const T *B)
 {
+    if constexpr (sizeof(T) == 8) {
+        if (!B && nc >= kSplitMinResid)
+            return launch_split_coarse_rhs(vc, fc, m_fine, c_coarse, nc, cfc, st);
+    }
     const long long work = (long long)nc * nc * nc;
     if (B)
         k_coarse_rhs<T, true><<<grid_spread(work), block_spread(work), 0, st>>>(vc, fc, m_fine, c_coarse, nc, cfc, B);
@@ -1146,6 +1160,8 @@ cudaError_t launch_patch_sweep(const double *in, double *out, const double *fint
 {
     if ((pf[0] | pf[1] | pf[2]) & 1)
         return cudaErrorInvalidValue;   // the pair mapping needs even sides
+    if (!mask && !v0 && (long long)pf[0] * pf[1] * pf[2] >= kSplitMinPatch)
+        return launch_split_patch_sweep(in, out, fint, rhs_add, pf, cf, clamp, st);
     const long long work = (long long)pf[0] * pf[1] * (pf[2] / 2);
     const int bs = block_spread(work), g = grid_spread(work);
     const bool split = !mask && v0;

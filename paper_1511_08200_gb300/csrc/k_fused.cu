@@ -323,6 +323,8 @@ cudaError_t prepare_fused_kernels()
         e = prepare_march_kernel();
     if (e == cudaSuccess)
         e = prepare_resid_march_kernel();
+    if (e == cudaSuccess)
+        e = prepare_split_kernels();
     return e;
 }
 

@@ -477,6 +477,8 @@ cudaError_t launch_pbox_resid_restrict(const double *v, const double *f, const i
                                        const unsigned char *mask, const Fin &fin)
 {
     const long long work = (long long)(p[0] / 2) * (p[1] / 2) * (p[2] / 2);
+    if (!mask && 8 * work >= kSplitMinPatch)
+        return launch_split_patch_resid_restrict(v, f, p, cf, vc, v0c, fc, partials, nblocks, st, fin);
     int g;
     if (8 * work <= kChildMaxFine) {   // a thread per fine cell
         const int bs = block_spread(8 * work);

@@ -221,6 +221,35 @@ cudaError_t launch_coarsest(T *v, T *tmp, const T *f, int n, CoefT<T> cf, double
                             double rtol, unsigned long long *clamp, int *sweeps, cudaStream_t st,
                             const T *B = nullptr);
 
+// ---- FP64 kernels in split arithmetic (k_split.cu, mg5_split.cuh)
+// Smaller sides keep the plain FP64 kernels.  Sweeps: a 48^3 half-sweep takes 4.0 us against 6.5, a
+// 32^3 solve lost 4% (16 tiles).  Residuals: 64^3 takes 12.3 us against 26.6, and below 64^3 the
+// FP64 residual is the more exact one (the stopping test is made of it).
+constexpr int kSplitMinSweep = 48, kSplitMinResid = 64;
+constexpr long long kSplitMinPatch = 40 * 40 * 40;   // cells of a patch's finest grid
+cudaError_t prepare_split_kernels();
+// snapshot red-black sweep (two launches), as launch_sweep
+cudaError_t launch_split_sweep(const double *in, double *out, const double *f, const double *cptr, int n,
+                               const CoefT<double> &cf, unsigned long long *clamp,
+                               cudaStream_t st);
+// the finest grid of a patch: as launch_patch_sweep without v0 and mask
+cudaError_t launch_split_patch_sweep(const double *in, double *out, const double *f, double add, const int p[3],
+                                     const CoefT<double> &cf, unsigned long long *clamp,
+                                     cudaStream_t st);
+cudaError_t launch_split_resid_restrict(const double *v, const double *f, const double *cptr, int n,
+                                        const CoefT<double> &cf, double *vc, double *v0c,
+                                        double *rc, double2 *partials, int *nblocks, cudaStream_t st, const Fin &fin);
+cudaError_t launch_split_residual(const double *v, const double *f, const double *cptr, int n,
+                                  const CoefT<double> &cf, double *r, double2 *partials,
+                                  int *nblocks, cudaStream_t st, const Fin &fin);
+// f = op(v) + f - m_fine; c_coarse = 0
+cudaError_t launch_split_coarse_rhs(const double *v, double *f, const double *m_fine, double *c_coarse, int n,
+                                    const CoefT<double> &cf, cudaStream_t st);
+cudaError_t launch_split_patch_resid_restrict(const double *v, const double *f, const int p[3],
+                                              const CoefT<double> &cf, double *vc,
+                                              double *v0c, double *fc, double2 *partials, int *nblocks,
+                                              cudaStream_t st, const Fin &fin);
+
 // ---- FP64 helpers
 cudaError_t launch_finalize(const double2 *partials, int nb, double ncells, LevelScal *ls,
                             int mode, cudaStream_t st);
