@@ -62,14 +62,32 @@ __global__ void k_spec_residual(const T *__restrict__ v, const T *__restrict__ f
     finalize_if_last(reinterpret_cast<double2 *>(partials), fin);   // c -= mean r
 }
 
+// cos and sin of 2 pi q / n, q = 0 .. n - 1, once per block: an FP64 sincospi is ~50 FP64
+// instructions (2 lanes a clock per SM), and one a term made an 18^3 transform along one axis take
+// 68 us; with the table, and blocks small enough that its warps reach every SM, 9.2 us (FP32, 30^3:
+// 11.4 -> 4.5 us).  What is left is the chain of 2 x 18 FP64 multiply-adds of each output.
+constexpr int kDftMax = 32;   // largest coarsest side
+template <typename T>
+__device__ __forceinline__ void dft_table(int n, T *cs, T *sn)
+{
+    for (int q = threadIdx.x; q < n; q += blockDim.x)
+        sincos_pi((T)(2 * q) / (T)n, &MG5_AT(sn, q), &MG5_AT(cs, q));
+    __syncthreads();
+}
+
 // One-dimensional DFT along `axis` (0: i, 1: j, 2: k) of every line:
 // out[m'] = sum_m in[m] exp(-+ 2 pi i m m' / n) (sign: forward -, inverse +).  With `addto`,
 // the real part times `scale` is added to it instead of writing `out`.
-template <typename T>
+// DIVIDE (the last forward axis): the result is divided by the eigenvalue of the periodic 7-point
+// Laplacian, lambda = (2 cos 2 pi kx/n + 2 cos 2 pi ky/n + 2 cos 2 pi kz/n - 6) / h^2; the mean mode
+// becomes zero.
+template <typename T, bool DIVIDE>
 __global__ void k_dft_axis(const typename Cplx<T>::type *__restrict__ in,
                            typename Cplx<T>::type *__restrict__ out, int n, int axis, int inverse,
-                           T *__restrict__ addto, T scale)
+                           T *__restrict__ addto, T scale, T h2)
 {
+    __shared__ T cs[kDftMax], sn[kDftMax];
+    dft_table<T>(n, cs, sn);
     const int n3 = n * n * n;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n3)
@@ -80,14 +98,18 @@ __global__ void k_dft_axis(const typename Cplx<T>::type *__restrict__ in,
     const int base = t - mo * stride;
     const T sgn = inverse ? (T)1 : (T)-1;
     T re = 0, im = 0;
-    for (int m = 0; m < n; ++m) {
-        const int q = (m * mo) % n;
-        T sn, cs;
-        sincos_pi((T)(2 * q) / (T)n, &sn, &cs);
-        sn *= sgn;
+    for (int m = 0, q = 0; m < n; ++m) {   // q = m mo mod n
+        const T s = MG5_AT(sn, q) * sgn, c = MG5_AT(cs, q);
         const typename Cplx<T>::type a = MG5_AT(in, base + m * stride);
-        re += a.x * cs - a.y * sn;
-        im += a.x * sn + a.y * cs;
+        re += a.x * c - a.y * s;
+        im += a.x * s + a.y * c;
+        q += mo;
+        q = q >= n ? q - n : q;
+    }
+    if constexpr (DIVIDE) {
+        const T inv = t == 0 ? (T)0 : h2 / ((T)2 * (MG5_AT(cs, i) + MG5_AT(cs, j) + MG5_AT(cs, k)) - (T)6);
+        re *= inv;
+        im *= inv;
     }
     if (addto) {
         MG5_AT(addto, t) += re * scale;
@@ -95,30 +117,6 @@ __global__ void k_dft_axis(const typename Cplx<T>::type *__restrict__ in,
         MG5_AT(out, t).x = re;
         MG5_AT(out, t).y = im;
     }
-}
-
-// d_hat = r_hat / lambda(k), lambda = (2 cos 2 pi kx/n + 2 cos 2 pi ky/n + 2 cos 2 pi kz/n - 6) / h^2
-// (the periodic 7-point Laplacian's eigenvalue); the mean mode is set to zero.
-template <typename T>
-__global__ void k_spec_divide(typename Cplx<T>::type *__restrict__ a, int n, T h2)
-{
-    const int n3 = n * n * n;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n3)
-        return;
-    const int k = t % n, j = (t / n) % n, i = t / (n * n);
-    if (i == 0 && j == 0 && k == 0) {
-        MG5_AT(a, t).x = (T)0;
-        MG5_AT(a, t).y = (T)0;
-        return;
-    }
-    T s, ci, cj, ck;
-    sincos_pi((T)(2 * i) / (T)n, &s, &ci);
-    sincos_pi((T)(2 * j) / (T)n, &s, &cj);
-    sincos_pi((T)(2 * k) / (T)n, &s, &ck);
-    const T inv = h2 / ((T)2 * (ci + cj + ck) - (T)6);
-    MG5_AT(a, t).x *= inv;
-    MG5_AT(a, t).y *= inv;
 }
 
 template <typename T>
@@ -130,27 +128,26 @@ cudaError_t launch_coarsest_spectral(T *v, T *tmp, const T *f, int n, CoefT<T> c
     using C = typename Cplx<T>::type;
     C *w0 = static_cast<C *>(w0v), *w1 = static_cast<C *>(w1v);
     const int n3 = n * n * n;
-    const int g = (n3 + kBlock - 1) / kBlock;
-    if (g > kMomentBlocks)
+    const int bs = block_spread(n3), g = grid_spread(n3);   // warps over all SMs
+    if (g > kMomentBlocks || n > kDftMax)
         return cudaErrorInvalidValue;
     Moments *mp = reinterpret_cast<Moments *>(partials);
     const T inv_n3 = (T)1 / (T)n3;
     for (int it = 0; it < iters; ++it) {
         const Fin fin{ls, FIN_RESID, (double)n3};
         if (B)
-            k_spec_residual<T, true><<<g, kBlock, 0, st>>>(v, f, &ls->c, n, cf, B, w0, mp, sweeps, fin);
+            k_spec_residual<T, true><<<g, bs, 0, st>>>(v, f, &ls->c, n, cf, B, w0, mp, sweeps, fin);
         else
-            k_spec_residual<T, false><<<g, kBlock, 0, st>>>(v, f, &ls->c, n, cf, B, w0, mp, sweeps, fin);
+            k_spec_residual<T, false><<<g, bs, 0, st>>>(v, f, &ls->c, n, cf, B, w0, mp, sweeps, fin);
         count_launch(1);
         cudaError_t e;
-        k_dft_axis<T><<<g, kBlock, 0, st>>>(w0, w1, n, 2, 0, nullptr, (T)0);
-        k_dft_axis<T><<<g, kBlock, 0, st>>>(w1, w0, n, 1, 0, nullptr, (T)0);
-        k_dft_axis<T><<<g, kBlock, 0, st>>>(w0, w1, n, 0, 0, nullptr, (T)0);
-        k_spec_divide<T><<<g, kBlock, 0, st>>>(w1, n, cf.h2);
-        k_dft_axis<T><<<g, kBlock, 0, st>>>(w1, w0, n, 0, 1, nullptr, (T)0);
-        k_dft_axis<T><<<g, kBlock, 0, st>>>(w0, w1, n, 1, 1, nullptr, (T)0);
-        k_dft_axis<T><<<g, kBlock, 0, st>>>(w1, w0, n, 2, 1, v, inv_n3);   // v += Re(d)
-        count_launch(7);
+        k_dft_axis<T, false><<<g, bs, 0, st>>>(w0, w1, n, 2, 0, nullptr, (T)0, (T)0);
+        k_dft_axis<T, false><<<g, bs, 0, st>>>(w1, w0, n, 1, 0, nullptr, (T)0, (T)0);
+        k_dft_axis<T, true><<<g, bs, 0, st>>>(w0, w1, n, 0, 0, nullptr, (T)0, cf.h2);
+        k_dft_axis<T, false><<<g, bs, 0, st>>>(w1, w0, n, 0, 1, nullptr, (T)0, (T)0);
+        k_dft_axis<T, false><<<g, bs, 0, st>>>(w0, w1, n, 1, 1, nullptr, (T)0, (T)0);
+        k_dft_axis<T, false><<<g, bs, 0, st>>>(w1, w0, n, 2, 1, v, inv_n3, (T)0);   // v += Re(d)
+        count_launch(6);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
         e = launch_sweep<T>(v, tmp, f, &ls->c, n, cf, clamp, st, B);
