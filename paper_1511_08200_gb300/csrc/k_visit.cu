@@ -1,0 +1,862 @@
+// k_visit.cu -- the coarse part of an FP64 V-cycle in one thread-block cluster: the visit of a
+// coarse grid of up to ~32^3 cells and of every grid below it (FAS right-hand side, nu1 snapshot
+// red-black sweeps, residual and 8-child restriction, ..., the coarsest iteration, ..., trilinear
+// prolongation of the correction, nu2 sweeps; Sec. 3.1), for periodic grids and for the Dirichlet
+// patch hierarchy.
+//
+// What bounds the level-by-level launches there is latency: 3 .. 12 us each for a few hundred ns of
+// work, and FP64 at 2 lanes a clock per SM.  One kernel keeps every grid in shared memory:
+//  * the planes of a grid are dealt to the 16 CTAs; grids of up to 8 planes or 512 cells and the
+//    coarsest one live in CTA 0, where a barrier costs less than a cluster one and the cells still
+//    fit the threads;
+//  * a value is its three FP32 pieces (mg5_split.cuh) on a unit fixed per grid and visit (the grid's
+//    largest exponent, the size a correction can have, and two bits): the stencil is exact, an update
+//    is a pair added to the pieces, rounded to 2^-58 of the largest value, and no FP64 instruction is
+//    left in a sweep.  Three arrays hold the two colours and the one being written (a half-sweep reads
+//    the old values of its own colour at the edges), 16 bytes a cell; a CTA's planes have copies of
+//    their neighbours' planes beside them, which the neighbours write through distributed shared
+//    memory as they update;
+//  * the residual, its restriction and the correction pass between grids as pairs through the grids'
+//    own global buffers (L2);
+//  * a value that outgrows its unit raises a flag: at the end all CTAs agree and repeat the visit
+//    with eight bits more.
+//
+// The FAS right-hand side is formed by the same pair arithmetic as the residual (relative 2^-47); the
+// corrections it leads to vanish with the residual, so the V-cycles converge as before.
+#include <cooperative_groups.h>
+
+#include "mg5_fin.cuh"
+#include "mg5_split.cuh"
+#include "mg5_visit.cuh"
+
+namespace mg5 {
+
+namespace cg = cooperative_groups;
+using namespace split::one;
+using split::Kap;
+using split::kUnitBias;
+
+namespace {
+
+constexpr int VT = 512;                 // threads
+constexpr float kPieceMax = 1048576.0f; // 2^20: sums of 12 pieces stay exact
+constexpr int kRestarts = 6;
+
+__device__ __forceinline__ int div_by(int t, unsigned m) { return m ? (int)__umulhi((unsigned)t, m) : t; }
+
+struct LevelState {
+    int eb;
+    Pr c;      // compatibility constant, units u / h^2
+    Kap kap;
+};
+
+struct VisitShared {
+    LevelState st[kVisitLevels];
+    int ebs[kVisitCtas];
+    Pr sums[kVisitCtas];
+    Pr red[2][VT / 32];
+    Pr bc[2];
+    int emax;
+    int flags[kVisitCtas];
+    int flag;
+};
+
+__device__ __forceinline__ double pow2d(int e) { return __hiloint2double((e + 1023) << 20, 0); }
+__device__ __forceinline__ Pr shfl_down(const Pr &x, int q)
+{
+    return Pr{__shfl_down_sync(0xffffffffu, x.h, q), __shfl_down_sync(0xffffffffu, x.l, q)};
+}
+__device__ __forceinline__ float pow2f(int e)
+{
+    e = e < -126 ? -126 : (e > 127 ? 127 : e);
+    return __int_as_float((e + 127) << 23);
+}
+__device__ __forceinline__ Pr pair_at(double x, int k)
+{
+    return pair_scaled((unsigned)__double2hiint(x), (unsigned)__double2loint(x), k);
+}
+// (x) 2^(eb - kUnitBias) as a double
+__device__ __forceinline__ double to_f64(const Pr &x, int eb)
+{
+    unsigned h0, l0, h1, l1;
+    split::unit_words(x.h, eb, h0, l0);
+    split::unit_words(x.l, eb, h1, l1);
+    const double d = __hiloint2double((int)h0, (int)l0) + __hiloint2double((int)h1, (int)l1);
+    return fabsf(x.h) < 1e30f ? d : __longlong_as_double(0x7ff8000000000000ll);
+}
+
+// One visit.  Positions: p a plane of this CTA counted from its first one (-1 and np: the copies of the
+// neighbours' planes, or a box's ghost planes), i = i0 + p; interior cells j, k.
+template <bool BOX>
+struct Visit {
+    const VisitArgs &A;
+    VisitShared &S;
+    float4 *sm;
+    cg::cluster_group cluster;
+    int rank, tid;
+    unsigned clamps = 0;
+    int sweeps = 0;
+
+    // the planes [i0, i0 + np) of level l this CTA owns
+    struct Own {
+        int i0, np;
+    };
+    __device__ __forceinline__ Own own(const VisitLevel &L, int r) const
+    {
+        if (L.single)
+            return Own{0, r == 0 ? L.n0 : 0};
+        const int i0 = r * L.P, np = min(L.n0 - i0, L.P);
+        return Own{i0, np > 0 ? np : 0};
+    }
+    __device__ __forceinline__ void bar(const VisitLevel &L)
+    {
+        if (L.single)
+            __syncthreads();
+        else
+            cluster.sync();
+    }
+    // Three arrays hold the two colours and the one a half-sweep writes, in turn: after b sweeps
+    // (mod 3) colour 0 is array (3 - b) % 3, colour 1 (4 - b) % 3 and the free one (5 - b) % 3.
+    static __device__ __forceinline__ int mod3(int x) { return x >= 3 ? x - 3 : x; }
+    static __device__ __forceinline__ int arr(int colour, int b) { return mod3(3 + colour - b); }
+    // a place in an array: a box keeps its ghost shell, a periodic grid wraps its indices; planes have
+    // their neighbours on both sides unless CTA 0 holds the whole periodic grid
+    __device__ __forceinline__ int at(const VisitLevel &L, int p, int j, int k) const
+    {
+        return BOX ? ((p + 1) * (L.n1 + 2) + j + 1) * L.wq + ((k + 1) >> 1)
+                   : ((p + 1 - L.single) * L.n1 + j) * L.wq + (k >> 1);
+    }
+    __device__ __forceinline__ float4 *array(const VisitLevel &L, int a) const { return sm + L.pieces + a * L.sz; }
+    static __device__ __forceinline__ P1 ld(const float4 &x) { return P1{x.x, x.y, x.z}; }
+    static __device__ __forceinline__ float4 st(const P1 &x) { return make_float4(x.h, x.m, x.l, 0.0f); }
+    // Interior cell into array a, and into the neighbours' copies of its plane.
+    __device__ __forceinline__ void put(const VisitLevel &L, const Own &o, int a, int p, int j, int k, const P1 &x)
+    {
+        const float4 v = st(x);
+        const int q = at(L, p, j, k);
+        array(L, a)[q] = v;
+        if (L.single)
+            return;
+        const int ps = (BOX ? L.n1 + 2 : L.n1) * L.wq;
+        if (p == 0 && (!BOX || rank > 0)) {
+            const int r = rank == 0 ? L.act - 1 : rank - 1;
+            cluster.map_shared_rank(array(L, a), r)[q + own(L, r).np * ps] = v;
+        }
+        if (p == o.np - 1 && (!BOX || rank < L.act - 1)) {
+            const int r = rank == L.act - 1 ? 0 : rank + 1;
+            cluster.map_shared_rank(array(L, a), r)[q - o.np * ps] = v;
+        }
+    }
+    // The stencil of cell (p, j, k): centre and edges from array ac, faces from array ao.
+    __device__ __forceinline__ Lin1 lin_at(const VisitLevel &L, int ac, int ao, int p, int j, int k) const
+    {
+        const int ps = (BOX ? L.n1 + 2 : L.n1) * L.wq, row = L.wq;
+        int xp = ps, xm = -ps, yp = row, ym = -row, zp, zm;
+        if (BOX) {
+            zp = (k + 1) & 1;
+            zm = zp - 1;
+        } else {
+            if (L.single) {
+                xp = p == L.n0 - 1 ? -(L.n0 - 1) * ps : ps;
+                xm = p == 0 ? (L.n0 - 1) * ps : -ps;
+            }
+            yp = j == L.n1 - 1 ? -(L.n1 - 1) * row : row;
+            ym = j == 0 ? (L.n1 - 1) * row : -row;
+            zp = k == L.n2 - 1 ? -(k >> 1) : (k & 1);
+            zm = k == 0 ? row - 1 : (k & 1) - 1;
+        }
+        const int q = at(L, p, j, k);
+        const float4 *a = array(L, ac) + q, *b = array(L, ao) + q;
+        const auto Av = [&](int x) { return ld(a[x]); };
+        const auto Ov = [&](int x) { return ld(b[x]); };
+        return lin_of(Av(0), Ov(xp) + Ov(xm), Ov(yp) + Ov(ym), Ov(zp) + Ov(zm),
+                      (Av(xp + yp) - Av(xp + ym)) - (Av(xm + yp) - Av(xm + ym)),
+                      (Av(xp + zp) - Av(xp + zm)) - (Av(xm + zp) - Av(xm + zm)),
+                      (Av(yp + zp) - Av(yp + zm)) - (Av(ym + zp) - Av(ym + zm)));
+    }
+    __device__ __forceinline__ P1 centre(const VisitLevel &L, int b, int p, int j, int k, int colour) const
+    {
+        return ld(array(L, arr(colour, b))[at(L, p, j, k)]);
+    }
+    __device__ __forceinline__ float2 &Fat(const VisitLevel &L, int p, int j, int k) const
+    {
+        return reinterpret_cast<float2 *>(sm + L.F)[(p * L.n1 + j) * L.n2 + k];
+    }
+    __device__ __forceinline__ Pr Fget(const VisitLevel &L, int p, int j, int k) const
+    {
+        const float2 f = Fat(L, p, j, k);
+        return Pr{f.x, f.y};
+    }
+    // every interior cell (p, j, k) of this CTA
+    template <typename F>
+    __device__ __forceinline__ void cells(const VisitLevel &L, const Own &o, const F &f)
+    {
+        const int n = o.np * L.n1 * L.n2;
+#pragma unroll 1
+        for (int t = tid; t < n; t += VT) {
+            const int q = div_by(t, L.m2), k = t - q * L.n2, p = div_by(q, L.m1), j = q - p * L.n1;
+            f(p, j, k);
+        }
+    }
+    __device__ __forceinline__ long long gcell(const VisitLevel &L, int i, int j, int k) const
+    {
+        return ((long long)i * L.n1 + j) * L.n2 + k;
+    }
+    // a cell's place in the level's v0 and v (box: with its ghost shell)
+    __device__ __forceinline__ long long vcell(const VisitLevel &L, int i, int j, int k) const
+    {
+        return BOX ? ((long long)(i + 1) * (L.n1 + 2) + j + 1) * (L.n2 + 2) + k + 1 : gcell(L, i, j, k);
+    }
+    __device__ __forceinline__ double v0_at(const VisitLevel &L, int i, int j, int k) const
+    {
+        return __ldcg(&MG5_AT(L.v0, vcell(L, i, j, k)));
+    }
+    // h^2 x / u as a pair
+    __device__ __forceinline__ Pr in_units(const VisitLevel &L, double x, int eb) const
+    {
+        return mul_pair(pair_at(x, kUnitBias - eb + L.Hq), Pr{L.Hh, L.Hl});
+    }
+    static __device__ __forceinline__ P1 split_f64(double x, int eb)
+    {
+        return split1((unsigned)__double2hiint(x), (unsigned)__double2loint(x), eb);
+    }
+    // the change of a cell since the visit began
+    __device__ __forceinline__ Pr change(const P1 &now, double v0, int eb) const
+    {
+        return pair_of(now - split_f64(v0, eb));
+    }
+
+    // ---- a box's ghosts: v0(g) + w^m (v(a) - v0(a)), a the nearest interior cell, m axes outside
+    struct Ghost {
+        int p, j, k, m;       // its place
+        int pa, ja, ka, ca;   // the interior cell and its colour
+    };
+    // Ghost number t of this CTA: the rings around its planes and their two neighbours, then the
+    // insides of a ghost plane.
+    __device__ __forceinline__ int ghost_count(const VisitLevel &L, const Own &o) const
+    {
+        if (!BOX || o.np == 0)
+            return 0;
+        const int ends = (o.i0 == 0) + (o.i0 + o.np == L.n0);
+        return (o.np + 2) * L.ring + ends * L.n1 * L.n2;
+    }
+    __device__ __forceinline__ Ghost ghost(const VisitLevel &L, const Own &o, int t) const
+    {
+        Ghost g;
+        const int rings = (o.np + 2) * L.ring;
+        if (t < rings) {
+            const int pl = div_by(t, L.mring), r = t - pl * L.ring, row = L.n2 + 2;
+            g.p = pl - 1;
+            if (r < 2 * row) {
+                g.j = r < row ? -1 : L.n1;
+                g.k = (r < row ? r : r - row) - 1;
+            } else {
+                g.j = (r - 2 * row) >> 1;
+                g.k = (r & 1) ? L.n2 : -1;   // 2 row is even
+            }
+        } else {
+            const int inside = L.n1 * L.n2;
+            int u = t - rings;
+            const bool second = u >= inside || o.i0 != 0;
+            if (u >= inside)
+                u -= inside;
+            g.p = second ? o.np : -1;
+            g.j = div_by(u, L.m2);
+            g.k = u - g.j * L.n2;
+        }
+        const int i = o.i0 + g.p, ia = min(max(i, 0), L.n0 - 1);
+        g.ja = min(max(g.j, 0), L.n1 - 1);
+        g.ka = min(max(g.k, 0), L.n2 - 1);
+        g.pa = ia - o.i0;
+        g.m = (i != ia) + (g.j != g.ja) + (g.k != g.ka);
+        g.ca = (ia + g.ja + g.ka) & 1;
+        return g;
+    }
+    __device__ __forceinline__ Pr weight(const VisitLevel &L, int m) const { return Pr{L.w[m - 1][0], L.w[m - 1][1]}; }
+    struct GhostBase {
+        double g, a;   // v0 of the ghost and of its cell
+    };
+    __device__ __forceinline__ GhostBase ghost_base(const VisitLevel &L, const Own &o, const Ghost &g) const
+    {
+        return GhostBase{v0_at(L, o.i0 + g.p, g.j, g.k), v0_at(L, o.i0 + g.pa, g.ja, g.ka)};
+    }
+    // The ghosts after a half-sweep (k_patch_half's order): after the red one every ghost of the
+    // sweep's result, after the black one those of the black cells.  a0, a1: the arrays of the two
+    // colours' values; d0, d1: of the ghosts.  first: the bases of ghost number tid.
+    __device__ __forceinline__ void ghosts_follow(const VisitLevel &L, const Own &o, bool black, int a0, int a1,
+                                                  int d0, int d1, const GhostBase &first, int eb)
+    {
+        const int n = ghost_count(L, o);
+#pragma unroll 1
+        for (int t = tid; t < n; t += VT) {
+            const Ghost g = ghost(L, o, t);
+            if (black && g.ca == 0)
+                continue;
+            const GhostBase v0 = t == tid ? first : ghost_base(L, o, g);
+            const P1 now = ld(array(L, g.ca ? a1 : a0)[at(L, g.pa, g.ja, g.ka)]);
+            const P1 x = add_change(split_f64(v0.g, eb), mul_pair(weight(L, g.m), change(now, v0.a, eb)));
+            array(L, (g.ca ^ (g.m & 1)) ? d1 : d0)[at(L, g.p, g.j, g.k)] = st(x);
+        }
+    }
+
+    // Level l from its parent's residual (the top one: from the caller's v), split; c = 0.
+    __device__ __forceinline__ void enter(const VisitLevel &L, int margin)
+    {
+        const Own o = own(L, rank);
+        if (tid == 0)
+            S.emax = 0;
+        __syncthreads();
+        int emax = 0;
+        const VisitLevel *U = L.id > 0 ? &A.lev[L.id - 1] : nullptr;
+        const int ebu = U ? S.st[U->id].eb : 0;
+        const int grow = L.nmax2 + L.Hq - 4;   // log2 of a correction's size over its residual's
+        cells(L, o, [&](int p, int j, int k) {
+            const int i = o.i0 + p;
+            double x;
+            if (U) {
+                double s = 0.0;
+                Pr r{0.0f, 0.0f};
+#pragma unroll
+                for (int ch = 0; ch < 8; ++ch) {
+                    const int fi = 2 * i + (ch >> 2), fj = 2 * j + ((ch >> 1) & 1), fk = 2 * k + (ch & 1);
+                    s += __ldcg(&MG5_AT(U->v, vcell(*U, fi, fj, fk)));
+                    const float2 q = __ldcg(&MG5_AT(U->x, gcell(*U, fi, fj, fk)));
+                    r = add_pair(r, Pr{q.x, q.y});
+                }
+                x = 0.125 * s;
+                MG5_AT(L.v0, vcell(L, i, j, k)) = x;
+                Fat(L, p, j, k) = make_float2(0.125f * r.h, 0.125f * r.l);
+                // r is in units of the parent's u / h^2
+                const int er = (int)((__float_as_uint(r.h) >> 23) & 0xffu);
+                if (er > 0)
+                    emax = max(emax, min(er - 127 - 3 + ebu - kUnitBias + 1023 - U->Hq + grow, 2046));
+            } else {
+                x = v0_at(L, i, j, k);
+                const int ef = (__double2hiint(MG5_AT(L.f, gcell(L, i, j, k))) >> 20) & 0x7ff;
+                if (ef > 0)
+                    emax = max(emax, min(ef + grow, 2046));
+            }
+            emax = max(emax, (__double2hiint(x) >> 20) & 0x7ff);
+        });
+        const int ng = ghost_count(L, o);
+        for (int t = tid; t < ng; t += VT) {   // the ghosts' fixed values
+            const Ghost g = ghost(L, o, t);
+            emax = max(emax, (__double2hiint(v0_at(L, o.i0 + g.p, g.j, g.k)) >> 20) & 0x7ff);
+        }
+        emax = __reduce_max_sync(0xffffffffu, emax);
+        if ((tid & 31) == 0)
+            atomicMax(&S.emax, emax);
+        __syncthreads();
+        if (!L.single) {
+            if (tid < kVisitCtas)
+                cluster.map_shared_rank(S.ebs, tid)[rank] = S.emax;
+            cluster.sync();
+            emax = 0;
+            for (int r = 0; r < kVisitCtas; ++r)
+                emax = max(emax, S.ebs[r]);
+        } else {
+            emax = S.emax;
+        }
+        const int eb = min(max((emax == 0 ? 1023 : emax) + margin, 200), 1800);
+        if (tid == 0) {
+            // (one thread: an FP64 instruction of every warp would take 256 clocks)
+            LevelState &st = S.st[L.id];
+            st.eb = eb;
+            st.c = Pr{0.0f, 0.0f};
+            const double k1 = L.k * pow2d(eb - kUnitBias), k3 = 3.0 * k1;
+            st.kap.k3h = (float)k3;
+            st.kap.k3l = (float)(k3 - (double)st.kap.k3h);
+            st.kap.kh = (float)k1;
+            st.kap.kl = (float)(k1 - (double)st.kap.kh);
+        }
+        cells(L, o, [&](int p, int j, int k) {
+            const int i = o.i0 + p;
+            put(L, o, arr((i + j + k) & 1, 0), p, j, k, split_f64(v0_at(L, i, j, k), eb));
+        });
+        for (int t = tid; t < ng; t += VT) {
+            const Ghost g = ghost(L, o, t);
+            array(L, arr(g.ca ^ (g.m & 1), 0))[at(L, g.p, g.j, g.k)] =
+                st(split_f64(v0_at(L, o.i0 + g.p, g.j, g.k), eb));
+        }
+        bar(L);
+    }
+
+    // The residual of every cell.  RHS: F = op(v) + R r - m of the parent, entering a grid.  DOWN: r and
+    // v for the restriction onto the next grid, sum of r.  TEST: sums of r and r^2 (c not counted).
+    enum Mode { RHS, DOWN, TEST };
+    __device__ __forceinline__ void residuals(const VisitLevel &L, int mode, int b, const Pr &Pm, Pr &sum, Pr &sq)
+    {
+        const Own o = own(L, rank);
+        const LevelState st = S.st[L.id];
+        const VisitLevel *U = L.id > 0 ? &A.lev[L.id - 1] : nullptr;
+        // from the parent's unit u / h^2: its h is half of L's
+        const float su = U ? 4.0f * pow2f(S.st[L.id - 1].eb - st.eb) : 0.0f;
+        Pr mean{0.0f, 0.0f};
+        if (!BOX && mode == RHS)
+            mean = U ? scale(Pm, su) : in_units(L, *A.m_up, st.eb);
+        sum = sq = Pr{0.0f, 0.0f};
+        cells(L, o, [&](int p, int j, int k) {
+            const int i = o.i0 + p, col = (i + j + k) & 1;
+            Pr F;
+            double v0 = 0.0;
+            if (mode == RHS) {
+                const Pr g = U ? scale(Fget(L, p, j, k), su) : in_units(L, MG5_AT(L.f, gcell(L, i, j, k)), st.eb);
+                F = add_pair(mean, neg(g));
+            } else {
+                F = Fget(L, p, j, k);
+                if (mode == DOWN) {
+                    v0 = v0_at(L, i, j, k);
+                    F = add_pair(F, st.c);
+                }
+            }
+            const Pr r = resid(lin_at(L, arr(col, b), arr(col ^ 1, b), p, j, k), F, st.kap);
+            if (mode == RHS) {
+                Fat(L, p, j, k) = make_float2(-r.h, -r.l);
+                return;
+            }
+            if (mode == DOWN) {
+                MG5_AT(L.x, gcell(L, i, j, k)) = make_float2(r.h, r.l);
+                // v = v0 + the change since then
+                MG5_AT(L.v, vcell(L, i, j, k)) = v0 + to_f64(change(centre(L, b, p, j, k, col), v0, st.eb), st.eb);
+            } else {
+                sq = add_pair(sq, sqr(r));
+            }
+            sum = add_pair(sum, r);
+        });
+    }
+
+    // One half-sweep: the cells of `colour` from array ac (faces from ao) into array ad.
+    __device__ __forceinline__ void half(const VisitLevel &L, const Own &o, int colour, int ac, int ao, int ad,
+                                         const Pr &c, const Kap &kap)
+    {
+        const int nq = (L.n2 + 1) >> 1, n = o.np * L.n1 * nq;
+#pragma unroll 1
+        for (int t = tid; t < n; t += VT) {
+            const int g = div_by(t, L.mq), q = t - g * nq, p = div_by(g, L.m1), j = g - p * L.n1;
+            const int k = 2 * q + ((o.i0 + p + j + colour) & 1);
+            if (k >= L.n2)
+                continue;
+            const Lin1 s = lin_at(L, ac, ao, p, j, k);
+            const Pr r = resid(s, add_pair(Fget(L, p, j, k), c), kap);
+            const Pr d = neg(mul_pair(root_change(s, r, kap, clamps), Pr{L.wh, L.wl}));
+            const P1 x = add_change(ld(array(L, ac)[at(L, p, j, k)]), d);
+            if (fabsf(x.h) > kPieceMax || fabsf(d.h) > 2.0f * kPieceMax)
+                S.flag = 1;
+            put(L, o, ad, p, j, k, x);
+        }
+    }
+    // `count` sweeps after b (mod 3); returns b + count (mod 3)
+    __device__ __forceinline__ int sweep(const VisitLevel &L, int count, int b)
+    {
+        const Own o = own(L, rank);
+        const LevelState st = S.st[L.id];
+        GhostBase first{0.0, 0.0};
+        if (tid < ghost_count(L, o))
+            first = ghost_base(L, o, ghost(L, o, tid));
+#pragma unroll 1
+        for (int s = 0; s < 2 * count; ++s) {
+            const int black = s & 1, a0 = arr(0, b), a1 = arr(1, b), free_ = mod3(5 - b);
+            // red: array a0 -> the free one; black: a1 -> what was a0
+            half(L, o, black, black ? a1 : a0, black ? free_ : a1, black ? a0 : free_, st.c, st.kap);
+            bar(L);
+            if (BOX) {
+                // red: the result's arrays are free_ (red) and a0 (black); black values still in a1
+                ghosts_follow(L, o, black, free_, black ? a0 : a1, free_, a0, first, st.eb);
+                __syncthreads();
+            }
+            if (black)
+                b = mod3(b + 1);
+        }
+        return b;
+    }
+    // Sums of two pairs over the CTA, in every thread (fixed order; in pair arithmetic: an FP64
+    // reduction of 16 warps would take over a microsecond).
+    __device__ __forceinline__ void block_sums(Pr &x, Pr &y)
+    {
+        for (int q = 16; q > 0; q >>= 1) {
+            x = add_pair(x, shfl_down(x, q));
+            y = add_pair(y, shfl_down(y, q));
+        }
+        if ((tid & 31) == 0) {
+            S.red[0][tid >> 5] = x;
+            S.red[1][tid >> 5] = y;
+        }
+        __syncthreads();
+        if (tid < 32) {
+            x = tid < VT / 32 ? S.red[0][tid] : Pr{0.0f, 0.0f};
+            y = tid < VT / 32 ? S.red[1][tid] : Pr{0.0f, 0.0f};
+            for (int q = VT / 64; q > 0; q >>= 1) {
+                x = add_pair(x, shfl_down(x, q));
+                y = add_pair(y, shfl_down(y, q));
+            }
+            if (tid == 0) {
+                S.bc[0] = x;
+                S.bc[1] = y;
+            }
+        }
+        __syncthreads();
+        x = S.bc[0];
+        y = S.bc[1];
+    }
+    // After the DOWN residuals: the mean residual (periodic), taken off c.
+    __device__ __forceinline__ Pr mean_residual(const VisitLevel &L, Pr sum)
+    {
+        Pr mean{0.0f, 0.0f}, none{0.0f, 0.0f};
+        if (BOX) {
+            bar(L);
+            return mean;
+        }
+        block_sums(sum, none);
+        if (!L.single && tid < kVisitCtas)
+            cluster.map_shared_rank(S.sums, tid)[rank] = sum;
+        bar(L);
+        if (!L.single) {
+            sum = S.sums[0];
+            for (int r = 1; r < L.act; ++r)
+                sum = add_pair(sum, S.sums[r]);
+        }
+        mean = mul_pair(sum, Pr{L.inv_h, L.inv_l});
+        if (tid == 0)
+            S.st[L.id].c = add_pair(S.st[L.id].c, neg(mean));
+        __syncthreads();
+        return mean;
+    }
+    // The correction since v0 as pairs, ghosts included, for the prolongation onto the grid above.
+    __device__ __forceinline__ void leave_up(const VisitLevel &L, int b)
+    {
+        const Own o = own(L, rank);
+        const int eb = S.st[L.id].eb;
+        cells(L, o, [&](int p, int j, int k) {
+            const int i = o.i0 + p;
+            const Pr e = change(centre(L, b, p, j, k, (i + j + k) & 1), v0_at(L, i, j, k), eb);
+            MG5_AT(L.x, vcell(L, i, j, k)) = make_float2(e.h, e.l);
+        });
+        const int ng = ghost_count(L, o);
+        for (int t = tid; t < ng; t += VT) {
+            const Ghost g = ghost(L, o, t);
+            const int i = o.i0 + g.p;
+            if (i >= 0 && i < L.n0 && (g.p < 0 || g.p >= o.np))
+                continue;   // a neighbour's plane
+            const Pr e = change(centre(L, b, g.pa, g.ja, g.ka, g.ca), v0_at(L, o.i0 + g.pa, g.ja, g.ka), eb);
+            const Pr w = mul_pair(weight(L, g.m), e);
+            MG5_AT(L.x, vcell(L, i, g.j, g.k)) = make_float2(w.h, w.l);
+        }
+    }
+    // v += P (correction of the grid below), c += its c
+    __device__ __forceinline__ void prolong(const VisitLevel &L, int b)
+    {
+        const Own o = own(L, rank);
+        const VisitLevel &D = A.lev[L.id + 1];
+        const int eb = S.st[L.id].eb, ebd = S.st[D.id].eb;
+        const float s64 = pow2f(ebd - eb) * (1.0f / 64.0f);
+        const auto three = [](const Pr &x, const Pr &y) {   // 3 x + y
+            const float p = mul(3.0f, x.h), e = fma(3.0f, x.h, -p);
+            const Pr s = two_sum(p, y.h);
+            return Pr{s.h, add(s.l, add(e, fma(3.0f, x.l, y.l)))};
+        };
+        cells(L, o, [&](int p, int j, int k) {
+            const int i = o.i0 + p, col = (i + j + k) & 1;
+            int a[3] = {i >> 1, j >> 1, k >> 1};
+            int n[3] = {(i & 1) ? a[0] + 1 : a[0] - 1, (j & 1) ? a[1] + 1 : a[1] - 1, (k & 1) ? a[2] + 1 : a[2] - 1};
+            if (!BOX) {
+                n[0] = n[0] < 0 ? D.n0 - 1 : (n[0] == D.n0 ? 0 : n[0]);
+                n[1] = n[1] < 0 ? D.n1 - 1 : (n[1] == D.n1 ? 0 : n[1]);
+                n[2] = n[2] < 0 ? D.n2 - 1 : (n[2] == D.n2 ? 0 : n[2]);
+            }
+            const auto E = [&](int x, int y, int z) {
+                const float2 q = __ldcg(&MG5_AT(D.x, vcell(D, x, y, z)));
+                return Pr{q.x, q.y};
+            };
+            const auto line = [&](int x, int y) { return three(E(x, y, a[2]), E(x, y, n[2])); };
+            const Pr y0 = three(line(a[0], a[1]), line(a[0], n[1])), y1 = three(line(n[0], a[1]), line(n[0], n[1]));
+            const Pr d = scale(three(y0, y1), s64);
+            const P1 x = add_change(centre(L, b, p, j, k, col), d);
+            if (fabsf(x.h) > kPieceMax || fabsf(d.h) > 2.0f * kPieceMax)
+                S.flag = 1;
+            put(L, o, arr(col, b), p, j, k, x);   // (a box's ghosts follow in the next sweep, as in k_patch_half)
+        });
+        if (!BOX) {
+            // c of the grid below from its unit u / h^2 (h^2 four times this one's)
+            const Pr c = add_pair(S.st[L.id].c, scale(S.st[D.id].c, 0.25f * pow2f(ebd - eb)));
+            __syncthreads();
+            if (tid == 0)
+                S.st[L.id].c = c;
+        }
+        bar(L);
+    }
+    // The coarsest grid's stopping rule (in CTA 0; as k_coarsest, k_pbox_coarsest): c = minus the mean
+    // residual; stop at rtol times the first norm.  r0: the first squared norm (negative: none yet).
+    __device__ __forceinline__ bool coarsest_done(const VisitLevel &L, Pr sum, Pr sq, float &r0)
+    {
+        block_sums(sum, sq);
+        if (!BOX) {
+            const Pr m = mul_pair(sum, Pr{L.inv_h, L.inv_l});
+            sq = add_pair(sq, neg(mul_pair(sum, m)));
+            if (tid == 0)
+                S.st[L.id].c = neg(m);
+            __syncthreads();
+        }
+        const float rn = sq.h > 0.0f ? sq.h : 0.0f;
+        if (r0 < 0.0f)
+            r0 = rn;
+        return rn <= (float)(A.rtol * A.rtol) * r0;
+    }
+
+    // One visit.  A loop over steps, so that the code of a residual pass and of a half-sweep exists
+    // once: inlined at each of their uses it outgrew the instruction cache (a half-sweep of 8^3 took
+    // 4400 clocks).
+    enum Step { ENTER, DOWNWARD, COARSEST, UPWARD, DONE };
+    __device__ __forceinline__ bool run(int margin)
+    {
+        if (tid == 0)
+            S.flag = 0;
+        cluster.sync();   // (also: every CTA of the cluster has started)
+        const int last = A.nlev - 1, bdn = A.nu1 % 3;   // bdn: the arrays' turn a grid is left in on the way down
+        int split_at = A.nlev;                          // first level held by CTA 0 alone
+        while (split_at > 0 && A.lev[split_at - 1].single)
+            --split_at;
+        int l = 0, b = 0, it = 0, step = ENTER;
+        float r0 = -1.0f;
+        Pr mean{0.0f, 0.0f};
+        if (split_at == 0 && rank != 0)
+            step = DONE;
+#pragma unroll 1
+        while (step != DONE) {
+            const VisitLevel &L = A.lev[l];
+            int count = 0;
+            if (step == UPWARD) {
+                if (l == split_at - 1) {
+                    // CTA 0's correction, with its unit and c, for the grid that the CTAs share
+                    if (rank == 0 && tid > 0 && tid < kVisitCtas)
+                        cluster.map_shared_rank(S.st, tid)[split_at] = S.st[split_at];
+                    cluster.sync();
+                }
+                prolong(L, bdn);
+                b = bdn;
+                count = A.nu2;
+            } else {
+                if (step == ENTER)
+                    enter(L, margin);
+                Pr sum, sq;
+                residuals(L, step == ENTER ? RHS : (step == DOWNWARD ? DOWN : TEST), step == ENTER ? 0 : b, mean, sum,
+                          sq);
+                if (step == ENTER) {
+                    __syncthreads();   // F, read by other threads in a sweep
+                    b = 0;
+                    if (l == last) {
+                        step = COARSEST;
+                        continue;
+                    }
+                    count = A.nu1;
+                } else if (step == DOWNWARD) {
+                    mean = mean_residual(L, sum);
+                    ++l;
+                    step = ENTER;
+                    if (A.lev[l].single && rank != 0) {
+                        l = split_at - 1;
+                        step = UPWARD;
+                    }
+                    continue;
+                } else {
+                    if (it < A.nu_coarse && !coarsest_done(L, sum, sq, r0)) {
+                        ++it;
+                        count = 1;
+                    } else {
+                        if (l > 0)
+                            leave_up(L, b);
+                        __syncthreads();
+                        step = l > 0 ? UPWARD : DONE;
+                        --l;
+                        continue;
+                    }
+                }
+            }
+            b = sweep(L, count, b);
+            if (step == ENTER) {
+                step = DOWNWARD;
+            } else if (step == UPWARD) {
+                if (l > 0) {
+                    leave_up(L, b);
+                    bar(L);
+                }
+                if (--l < 0 || (A.lev[l].single && rank != 0))
+                    step = DONE;
+            }
+        }
+        sweeps += it;
+        // agree on the flag
+        __syncthreads();
+        if (tid < kVisitCtas)
+            cluster.map_shared_rank(S.flags, tid)[rank] = S.flag;
+        cluster.sync();
+        int any = 0;
+        for (int r = 0; r < kVisitCtas; ++r)
+            any |= S.flags[r];
+        if (any && margin < 2 + 8 * kRestarts)
+            return false;
+        // the top grid's iterate and c
+        const VisitLevel &L = A.lev[0];
+        const Own o = own(L, rank);
+        const LevelState st = S.st[0];
+        cells(L, o, [&](int p, int j, int k) {
+            const int i = o.i0 + p;
+            const double v0 = v0_at(L, i, j, k);
+            MG5_AT(L.v, vcell(L, i, j, k)) =
+                v0 + to_f64(change(centre(L, b, p, j, k, (i + j + k) & 1), v0, st.eb), st.eb);
+        });
+        const int ng = ghost_count(L, o);
+        for (int t = tid; t < ng; t += VT) {
+            const Ghost g = ghost(L, o, t);
+            const int i = o.i0 + g.p;
+            if (i >= 0 && i < L.n0 && (g.p < 0 || g.p >= o.np))
+                continue;
+            const GhostBase v0 = ghost_base(L, o, g);
+            const Pr e = change(centre(L, b, g.pa, g.ja, g.ka, g.ca), v0.a, st.eb);
+            MG5_AT(L.v, vcell(L, i, g.j, g.k)) = v0.g + to_f64(mul_pair(weight(L, g.m), e), st.eb);
+        }
+        if (!BOX && rank == 0 && tid == 0)
+            *A.c_out = to_f64(st.c, st.eb) / L.h2;
+        return true;
+    }
+};
+
+template <bool BOX>
+__global__ void __launch_bounds__(VT, 1) k_visit(const __grid_constant__ VisitArgs A)
+{
+    extern __shared__ __align__(16) float4 visit_sm[];
+    __shared__ VisitShared S;
+    cg::cluster_group cluster = cg::this_cluster();
+    Visit<BOX> V{A, S, visit_sm, cluster, (int)cluster.block_rank(), (int)threadIdx.x};
+    for (int margin = 2;; margin += 8) {
+        V.clamps = 0;
+        V.sweeps = 0;
+        if (V.run(margin))
+            break;
+    }
+    if (V.clamps)
+        atomicAdd(&MG5_AT(A.clamp, 0), (unsigned long long)V.clamps);
+    if (V.rank == 0 && V.tid == 0 && A.sweeps)
+        atomicAdd(&MG5_AT(A.sweeps, 0), V.sweeps);
+    cluster.sync();   // no CTA leaves while another may still write to its shared memory
+}
+
+cudaLaunchConfig_t cluster_config(int smem, cudaStream_t st, cudaLaunchAttribute *at)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kVisitCtas);
+    cfg.blockDim = dim3(VT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = kVisitCtas;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+unsigned magic(int d) { return d < 2 ? 0u : (unsigned)((0x100000000ull + d - 1) / d); }
+
+}  // namespace
+
+static bool g_visit_fits = false;   // a cluster of kVisitCtas CTAs can be resident (set by the preparation)
+
+bool visit_plan(const int (*q)[3], int nlev, bool box, VisitArgs *A)
+{
+    if (!g_visit_fits || nlev < 1 || nlev > kVisitLevels)
+        return false;
+    int quads = 0;   // of 16 bytes
+    for (int l = 0; l < nlev; ++l) {
+        VisitLevel &L = A->lev[l];
+        L.id = l;
+        L.n0 = q[l][0];
+        L.n1 = q[l][1];
+        L.n2 = q[l][2];
+        const long long cells = (long long)L.n0 * L.n1 * L.n2;
+        const bool tail = l == nlev - 1;
+        if (L.n0 < 2 || L.n1 < 2 || L.n2 < 2 || cells > 65536 || (tail && cells > kVisitCoarsest))
+            return false;
+        if (!box && ((L.n0 | L.n1 | L.n2) & 1))
+            return false;
+        L.single = tail || L.n0 <= 8 || cells <= 512;
+        if (l > 0 && A->lev[l - 1].single)
+            L.single = 1;
+        L.P = L.single ? L.n0 : (L.n0 + kVisitCtas - 1) / kVisitCtas;
+        L.act = L.single ? 1 : (L.n0 + L.P - 1) / L.P;
+        L.wq = box ? (L.n2 + 3) / 2 : L.n2 / 2;
+        L.sz = (box || !L.single ? L.P + 2 : L.P) * (box ? L.n1 + 2 : L.n1) * L.wq;
+        L.pieces = quads;
+        quads += 3 * L.sz;
+        L.F = quads;
+        quads += (L.P * L.n1 * L.n2 + 1) / 2;
+        L.ring = 2 * (L.n2 + 2) + 2 * L.n1;
+        L.mring = magic(L.ring);
+        L.mq = magic((L.n2 + 1) / 2);
+        L.m1 = magic(L.n1);
+        L.m2 = magic(L.n2);
+        L.inv_h = (float)(1.0 / (double)cells);
+        L.inv_l = (float)(1.0 / (double)cells - (double)L.inv_h);
+        int m = L.n0 > L.n1 ? L.n0 : L.n1;
+        m = m > L.n2 ? m : L.n2;
+        L.nmax2 = 0;
+        while (m > 1) {
+            m >>= 1;
+            L.nmax2 += 2;
+        }
+    }
+    A->nlev = nlev;
+    A->smem = quads * 16;
+    return A->smem <= kVisitSmem;
+}
+
+void visit_level_consts(VisitLevel *L, const CoefT<double> &cf, double w)
+{
+    const split::Coef cs = split::make_split_coef(cf);
+    int ex = 0;
+    const double H = 2.0 * std::frexp(cf.h2, &ex);
+    L->h2 = cf.h2;
+    L->k = cf.k23 * cf.inv_h2;
+    L->Hq = ex - 1;
+    L->Hh = (float)H;
+    L->Hl = (float)(H - (double)L->Hh);
+    L->wh = cs.wh;
+    L->wl = cs.wl;
+    double p = 1.0;
+    for (int m = 0; m < 3; ++m) {
+        p *= w;
+        L->w[m][0] = (float)p;
+        L->w[m][1] = (float)(p - (double)L->w[m][0]);
+    }
+}
+
+cudaError_t prepare_visit_kernels()
+{
+    cudaError_t e = cudaSuccess;
+    bool fits = true;
+    for (const void *k : {(const void *)k_visit<false>, (const void *)k_visit<true>}) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kVisitSmem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaLaunchAttribute at;
+        cudaLaunchConfig_t cfg = cluster_config(kVisitSmem, nullptr, &at);
+        int n = 0;
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
+        fits = fits && n > 0;
+    }
+    if (e == cudaSuccess)
+        g_visit_fits = fits;
+    return e;
+}
+
+cudaError_t launch_visit(const VisitArgs &A, bool box, cudaStream_t st)
+{
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = cluster_config(A.smem, st, &at);
+    const cudaError_t e = box ? cudaLaunchKernelEx(&cfg, k_visit<true>, A) : cudaLaunchKernelEx(&cfg, k_visit<false>, A);
+    count_launch(1);
+    return e;
+}
+
+}  // namespace mg5

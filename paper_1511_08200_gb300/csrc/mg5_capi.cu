@@ -23,6 +23,7 @@
 #include "mg5_mixed.cuh"
 #include "mg5_pool.h"
 #include "mg5_prof.cuh"
+#include "mg5_visit.cuh"
 
 using namespace mg5;
 
@@ -649,11 +650,51 @@ struct Run64 {
         return MG5_OK;
     }
 
+    // The visit of grid l and every grid below it in one launch (k_visit.cu); false: not these grids.
+    // Sides up to 32: a 64^3 grid's planes do not fit 16 SMs, and its launches fill the GPU.
+    bool visit(int l, cudaError_t *e)
+    {
+        if (h->n[l] > 32 || h->n[h->nlev - 1] >= kSpectralMinSide)
+            return false;
+        VisitArgs A = {};
+        int q[kMaxLevels][3];
+        for (int k = l; k < h->nlev; ++k)
+            q[k - l][0] = q[k - l][1] = q[k - l][2] = h->n[k];
+        if (!visit_plan(q, h->nlev - l, false, &A))
+            return false;
+        ProfScope ps(&ctx->prof, PK_COARSEST64, st);
+        for (int k = l; k < h->nlev; ++k) {
+            VisitLevel &L = A.lev[k - l];
+            visit_level_consts(&L, make_coef<double>(hl[k], p->alpha, omega_of(p)), 0.0);
+            L.v = h->v[k];
+            L.v0 = h->v0[k];
+            L.f = h->f[k];
+            L.x = reinterpret_cast<float2 *>(h->tmp[k]);
+            if (k < h->nlev - 1)
+                cu += (long long)(p->nu1 + p->nu2) * h->n[k] * h->n[k] * h->n[k];
+        }
+        A.nu1 = p->nu1;
+        A.nu2 = p->nu2;
+        A.nu_coarse = p->nu_coarse;
+        A.rtol = kCoarseRtol;
+        A.m_up = m(l - 1);
+        A.c_out = c(l);
+        A.clamp = &cntb->clamped;
+        A.sweeps = &cntb->coarse_sweeps;
+        *e = launch_visit(A, false, st);
+        return true;
+    }
+
     // coarse-grid correction for level l-1, entered with v[l] = v0[l] = R v[l-1]
     // and f[l] = R r[l-1]
     int coarse_visit(int l)
     {
         mg5_ctx *ctx = this->ctx;
+        cudaError_t ev = cudaSuccess;
+        if (visit(l, &ev)) {
+            CK(ev);
+            return MG5_OK;
+        }
         const CoefT<double> cfc = make_coef<double>(hl[l], p->alpha);
         {
             ProfScope ps(&ctx->prof, PK_COARSE_RHS64, st, (double)(h->n[l]) * (h->n[l]) * (h->n[l]));
@@ -929,6 +970,8 @@ int mg5_create(mg5_ctx **out, int device, size_t budget)
         e = cudaEventCreateWithFlags(&ctx->evb, cudaEventBlockingSync | cudaEventDisableTiming);
     if (e == cudaSuccess)
         e = prepare_fused_kernels();
+    if (e == cudaSuccess)
+        e = prepare_visit_kernels();
     if (e != cudaSuccess) {
         cudaGetLastError();
         mg5_destroy(ctx);
@@ -1376,9 +1419,42 @@ struct RunPatch {
         return MG5_OK;
     }
 
+    // The visit of grid l and every grid below it in one launch (k_visit.cu), as for the periodic
+    // grids; masked relaxations keep the launches.
+    bool visit(int l, cudaError_t *e)
+    {
+        VisitArgs A = {};
+        if (mk[0] || (long long)int_cells(h->q[l]) > kVisitCells || !visit_plan(h->q + l, h->nlev - l, true, &A))
+            return false;
+        ProfScope ps(&ctx->prof, PK_COARSEST64, st);
+        for (int k = l; k < h->nlev; ++k) {
+            VisitLevel &L = A.lev[k - l];
+            visit_level_consts(&L, make_coef<double>(hl[k], p->alpha, omega_of(p)), ghost_w(k));
+            L.v = h->v[k];
+            L.v0 = h->v0[k];
+            L.f = h->f[k];
+            L.x = reinterpret_cast<float2 *>(h->tmp[k]);
+            if (k < h->nlev - 1)
+                cu += (long long)(p->nu1 + p->nu2) * (long long)int_cells(h->q[k]);
+        }
+        A.nu1 = p->nu1;
+        A.nu2 = p->nu2;
+        A.nu_coarse = p->nu_coarse;
+        A.rtol = kCoarseRtol;
+        A.clamp = &cntb->clamped;
+        A.sweeps = &cntb->coarse_sweeps;
+        *e = launch_visit(A, true, st);
+        return true;
+    }
+
     int coarse_visit(int l)
     {
         mg5_ctx *ctx = this->ctx;
+        cudaError_t ev = cudaSuccess;
+        if (visit(l, &ev)) {
+            CK(ev);
+            return MG5_OK;
+        }
         // v = v0 on entry, its ghosts reset to the fixed coarse values by the restriction
         CK(launch_pbox_coarse_rhs(h->v[l], h->f[l], h->q[l], make_coef<double>(hl[l], p->alpha), st));
         if (l == h->nlev - 1)

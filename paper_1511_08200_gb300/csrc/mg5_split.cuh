@@ -318,5 +318,164 @@ MG5_HD void step_of(const Pair &d, const Coef &c, float2 &p, float2 &e)
     e = fma2(both(c.wl), d.h, e);
 }
 
+// ---- one cell at a time ---------------------------------------------------------
+// The same arithmetic on single values (k_visit.cu: coarse grids, where a CTA has fewer cells
+// than threads).  There the pieces are the value itself: add_change adds a pair to them, rounded
+// to the grid u 2^-40, and leaves h an integer, |m| <= 1/2 and |l| <= 2^-21.
+namespace one {
+
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+#else
+inline float add(float a, float b) { return fadd_(a, b); }
+inline float sub(float a, float b) { return fsub(a, b); }
+inline float mul(float a, float b) { return fmul(a, b); }
+inline float fma(float a, float b, float c) { return std::fmaf(a, b, c); }
+#endif
+
+struct P1 {
+    float h, m, l;
+};
+struct Pr {
+    float h, l;
+};
+MG5_HD P1 operator+(const P1 &a, const P1 &b) { return P1{add(a.h, b.h), add(a.m, b.m), add(a.l, b.l)}; }
+MG5_HD P1 operator-(const P1 &a, const P1 &b) { return P1{sub(a.h, b.h), sub(a.m, b.m), sub(a.l, b.l)}; }
+MG5_HD P1 minus2(const P1 &s, const P1 &c)
+{
+    return P1{fma(-2.0f, c.h, s.h), fma(-2.0f, c.m, s.m), fma(-2.0f, c.l, s.l)};
+}
+MG5_HD Pr two_sum(float a, float b)
+{
+    const float s = add(a, b), t = sub(s, a);
+    return Pr{s, add(sub(a, sub(s, t)), sub(b, t))};
+}
+MG5_HD Pr pair_of(const P1 &p)
+{
+    const float s = add(p.h, p.m);
+    return Pr{s, add(sub(p.m, sub(s, p.h)), p.l)};
+}
+MG5_HD Pr add_pair(const Pr &a, const Pr &b)
+{
+    const Pr s = two_sum(a.h, b.h);
+    return Pr{s.h, add(s.l, add(a.l, b.l))};
+}
+MG5_HD Pr mul_pair(const Pr &x, const Pr &y)
+{
+    const float p = mul(x.h, y.h);
+    return Pr{p, fma(x.l, y.h, fma(x.h, y.l, fma(x.h, y.h, -p)))};
+}
+MG5_HD Pr sqr(const Pr &x)
+{
+    const float p = mul(x.h, x.h);
+    return Pr{p, fma(fma(2.0f, x.h, x.l), x.l, fma(x.h, x.h, -p))};
+}
+// a power of two times x
+MG5_HD Pr scale(const Pr &x, float s) { return Pr{mul(x.h, s), mul(x.l, s)}; }
+MG5_HD Pr neg(const Pr &x) { return Pr{-x.h, -x.l}; }
+
+// The double with words (hi, lo) times 2^k as a pair.
+MG5_HD Pr pair_scaled(unsigned hi, unsigned lo, int k)
+{
+    const int e = (int)((hi >> 20) & 0x7ffu);
+    const int x = e == 0 ? 0 : (e == 2047 ? 2047 : e + k);
+    const unsigned h2 = (hi & 0x800fffffu) | ((unsigned)(x < 0 ? 0 : (x > 2047 ? 2047 : x)) << 20);
+    Pr r;
+    pair_words(h2, lo, r.h, r.l);
+    return r;
+}
+MG5_HD P1 split1(unsigned hi, unsigned lo, int eb)
+{
+    float h, m, l, sg;
+    const int e = (int)((hi >> 20) & 0x7ffu);
+    piece_bits(hi, lo, eb < e ? e : eb, h, m, l, sg);   // (infinity, NaN: any value)
+    return P1{mul(sub(h, 8388608.0f), sg), mul(sub(m, 8.0f), sg), mul(sub(l, 7.62939453125e-06f), sg)};
+}
+
+struct Lin1 {
+    Pr lam, X, W, Y, Z, xy, xz, yz;
+};
+MG5_HD Lin1 lin_of(const P1 &c, const P1 &sx, const P1 &sy, const P1 &sz, const P1 &dxy, const P1 &dxz,
+                   const P1 &dyz)
+{
+    Lin1 r;
+    const P1 X = minus2(sx, c), Y = minus2(sy, c), Z = minus2(sz, c);
+    const P1 W = Y + Z;
+    r.lam = pair_of(X + W);
+    r.X = pair_of(X);
+    r.W = pair_of(W);
+    r.Y = pair_of(Y);
+    r.Z = pair_of(Z);
+    r.xy = pair_of(dxy);
+    r.xz = pair_of(dxz);
+    r.yz = pair_of(dyz);
+    return r;
+}
+// lambda + kappa3 P (h^2 op / u) subtracted from F, normalised
+MG5_HD Pr resid(const Lin1 &t, const Pr &F, const Kap &k)
+{
+    Pr d = add_pair(add_pair(sqr(t.xy), sqr(t.xz)), sqr(t.yz));
+    const Pr P = add_pair(add_pair(mul_pair(t.X, t.W), mul_pair(t.Y, t.Z)), scale(d, -0.0625f));
+    const Pr q = mul_pair(Pr{k.k3h, k.k3l}, P);
+    const Pr a = two_sum(F.h, -t.lam.h), b = two_sum(a.h, -q.h);
+    return two_sum(b.h, add(sub(F.l, t.lam.l), sub(add(a.l, b.l), q.l)));
+}
+// As split::root_change; a cell near the double root (or not finite) takes the closed form in
+// FP64, as the FP64 kernels do, and a negative discriminant is clamped and counted.
+MG5_HD Pr root_change(const Lin1 &t, const Pr &r, const Kap &k, unsigned &clamps)
+{
+    const Pr kap{k.kh, k.kl};
+    const Pr q0 = scale(mul_pair(kap, t.lam), 2.0f);
+    const Pr o = two_sum(1.0f, q0.h);
+    const Pr q{o.h, add(o.l, q0.l)};
+    const float D = fma(4.0f * k.kh, r.h, mul(q.h, q.h));
+    if (D >= 0.25f && D < 1e30f && q.h > 0.0f) {
+        const float rs = rsq(D);
+        const float d0 = mul(add(r.h, r.h), rcp(fma(D, rs, q.h)));
+        const float p = mul(q.h, d0), e = fma(q.l, d0, fma(q.h, d0, -p));
+        const float kd = mul(k.kh, d0), ek = fma(k.kl, d0, fma(k.kh, d0, -kd));
+        const float p2 = mul(kd, d0), e2 = fma(ek, d0, fma(kd, d0, -p2));
+        const Pr s1 = two_sum(r.h, -p), s2 = two_sum(s1.h, -p2);
+        const float rho = add(s2.h, sub(add(r.l, add(s1.l, s2.l)), add(e, e2)));
+        return Pr{d0, mul(rho, rs)};
+    }
+    const double lam = (double)t.lam.h + (double)t.lam.l, kd = (double)k.kh + (double)k.kl;
+    const double b = lam + kd * lam * lam + ((double)r.h + (double)r.l), disc = 1.0 + 4.0 * kd * b;
+    double L = 2.0 * b;
+    if (disc < 0.0)
+        ++clamps;
+    else
+        L = 2.0 * b / (1.0 + sqrt(disc));
+    const double d = L - lam;
+    const float dh = (float)d;
+    return Pr{dh, (float)(d - (double)dh)};
+}
+
+MG5_HD float round_to(float x, float magic) { return sub(add(x, magic), magic); }
+constexpr float kMagic0 = 12582912.0f;           // 1.5 2^23: to integers
+constexpr float kMagic1 = 12.0f;                 // 1.5 2^3: to multiples of 2^-20
+constexpr float kMagic2 = 1.1444091796875e-05f;  // 1.5 2^-17: to multiples of 2^-40
+
+MG5_HD P1 add_change(const P1 &c, const Pr &d)
+{
+    const float a = round_to(d.h, kMagic0);
+    const Pr s = two_sum(sub(d.h, a), d.l);
+    const float b = round_to(s.h, kMagic1);
+    const float t = round_to(add(sub(s.h, b), s.l), kMagic2);
+    P1 r{add(c.h, a), add(c.m, b), add(c.l, t)};
+    const float x = round_to(r.l, kMagic1);
+    r.l = sub(r.l, x);
+    r.m = add(r.m, x);
+    const float y = round_to(r.m, kMagic0);
+    r.m = sub(r.m, y);
+    r.h = add(r.h, y);
+    return r;
+}
+
+}  // namespace one
+
 }  // namespace split
 }  // namespace mg5

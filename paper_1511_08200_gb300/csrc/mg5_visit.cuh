@@ -1,0 +1,49 @@
+// mg5_visit.cuh -- arguments of the coarse-grid visit in one cluster (k_visit.cu).
+#pragma once
+#include "mg5_kernels.cuh"
+
+namespace mg5 {
+
+constexpr int kVisitCtas = 16;
+constexpr int kVisitLevels = 6;
+constexpr int kVisitCells = 40 * 32 * 32;    // cells of the largest patch grid taken
+constexpr int kVisitCoarsest = 2048;          // cells of a coarsest grid CTA 0 iterates
+constexpr int kVisitSmem = 222 * 1024;        // dynamic shared memory a CTA may use
+
+struct VisitLevel {
+    int id, n0, n1, n2;    // interior sides
+    int P, act, single;    // planes per CTA, CTAs that own planes, held by CTA 0 alone
+    int wq, sz;            // cells of a row of one colour, of an array
+    int pieces, F;         // offsets in shared memory (16 bytes)
+    int ring;              // ghosts around a plane (box)
+    unsigned mq, m1, m2, mring;   // reciprocals of (n2 + 1) / 2, n1, n2, ring
+    int nmax2;             // 2 floor(log2 of the largest side)
+    int Hq;                // h^2 = H 2^Hq
+    float Hh, Hl;
+    float wh, wl;          // omega / 6
+    float inv_h, inv_l;    // 1 / cells
+    float w[3][2];         // ghost weights w, w^2, w^3 (box)
+    double h2, k;          // k = (2 alpha / 3) / h^2
+    double *v, *v0;
+    const double *f;       // the top grid's restricted residual
+    float2 *x;             // scratch: residuals on the way down, corrections on the way up
+};
+
+struct VisitArgs {
+    int nlev, nu1, nu2, nu_coarse, smem;
+    double rtol;
+    const double *m_up;    // mean residual of the grid above (periodic)
+    double *c_out;         // c of the top grid (periodic)
+    unsigned long long *clamp;
+    int *sweeps;
+    VisitLevel lev[kVisitLevels];
+};
+
+// Fills sides, distribution and shared-memory layout; false: the grids do not fit.
+bool visit_plan(const int (*q)[3], int nlev, bool box, VisitArgs *A);
+// ... and a level's constants (w: extrapolation weight of a box's ghosts).
+void visit_level_consts(VisitLevel *L, const CoefT<double> &cf, double w);
+cudaError_t prepare_visit_kernels();
+cudaError_t launch_visit(const VisitArgs &A, bool box, cudaStream_t st);
+
+}  // namespace mg5
