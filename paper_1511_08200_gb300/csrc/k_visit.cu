@@ -1,5 +1,5 @@
 // k_visit.cu -- the coarse part of an FP64 V-cycle in one thread-block cluster: the visit of a
-// coarse grid of up to ~32^3 cells and of every grid below it (FAS right-hand side, nu1 snapshot
+// coarse grid of up to 20000 cells and of every grid below it (FAS right-hand side, nu1 snapshot
 // red-black sweeps, residual and 8-child restriction, ..., the coarsest iteration, ..., trilinear
 // prolongation of the correction, nu2 sweeps; Sec. 3.1), for periodic grids and for the Dirichlet
 // patch hierarchy.
@@ -9,7 +9,7 @@
 //  * the planes of a grid are dealt to the 16 CTAs; grids of up to 8 planes or 512 cells and the
 //    coarsest one live in CTA 0, where a barrier costs less than a cluster one and the cells still
 //    fit the threads;
-//  * a value is its three FP32 pieces (mg5_split.cuh) on a unit fixed per grid and visit (the grid's
+//  * a value is its three FP32 pieces (mg5_split.cuh) on a unit fixed for the visit (the top grid's
 //    largest exponent, the size a correction can have, and two bits): the stencil is exact, an update
 //    is a pair added to the pieces, rounded to 2^-58 of the largest value, and no FP64 instruction is
 //    left in a sweep.  Three arrays hold the two colours and the one being written (a half-sweep reads
@@ -20,6 +20,12 @@
 //    own global buffers (L2);
 //  * a value that outgrows its unit raises a flag: at the end all CTAs agree and repeat the visit
 //    with eight bits more.
+//
+// Measured on GB300 (a visit, launches -> cluster): top grid 16^3 periodic 130 -> 67 us, with the
+// 32^3 patch's 16^3 grid below it 100 -> 46 us.  A half-sweep takes 2.1 kclk at 4^3, 2.95 at 8^3 and 3.6
+// at 16^3: a chain of ~450 dependent instructions, and at 16^3 the cluster barrier.  Tried: two cells a
+// thread in packed or in interleaved arithmetic (slower: the packed instructions' latency; the code
+// outgrows the instruction cache).
 //
 // The FAS right-hand side is formed by the same pair arithmetic as the residual (relative 2^-47); the
 // corrections it leads to vanish with the residual, so the V-cycles converge as before.
@@ -41,21 +47,16 @@ namespace {
 constexpr int VT = 512;                 // threads
 constexpr float kPieceMax = 1048576.0f; // 2^20: sums of 12 pieces stay exact
 constexpr int kRestarts = 6;
+constexpr int kHold = 4;                // top-grid cells a thread holds in registers
 
 __device__ __forceinline__ int div_by(int t, unsigned m) { return m ? (int)__umulhi((unsigned)t, m) : t; }
 
-struct LevelState {
-    int eb;
-    Pr c;      // compatibility constant, units u / h^2
-    Kap kap;
-};
-
 struct VisitShared {
-    LevelState st[kVisitLevels];
+    Pr c[kVisitLevels];   // compatibility constants, units u / h^2 of their grids
+    Kap kap;              // of the top grid
     int ebs[kVisitCtas];
     Pr sums[kVisitCtas];
-    Pr red[2][VT / 32];
-    Pr bc[2];
+    Pr red[2][2][VT / 32];
     int emax;
     int flags[kVisitCtas];
     int flag;
@@ -96,6 +97,8 @@ struct Visit {
     int rank, tid;
     unsigned clamps = 0;
     int sweeps = 0;
+    int eb = 0;      // the visit's exponent: u = 2^(eb - kUnitBias)
+    int turn = 0;    // of the reduction buffers
 
     // the planes [i0, i0 + np) of level l this CTA owns
     struct Own {
@@ -212,18 +215,21 @@ struct Visit {
         return __ldcg(&MG5_AT(L.v0, vcell(L, i, j, k)));
     }
     // h^2 x / u as a pair
-    __device__ __forceinline__ Pr in_units(const VisitLevel &L, double x, int eb) const
+    __device__ __forceinline__ Pr in_units(const VisitLevel &L, double x) const
     {
         return mul_pair(pair_at(x, kUnitBias - eb + L.Hq), Pr{L.Hh, L.Hl});
     }
-    static __device__ __forceinline__ P1 split_f64(double x, int eb)
+    __device__ __forceinline__ P1 split_f64(double x) const
     {
         return split1((unsigned)__double2hiint(x), (unsigned)__double2loint(x), eb);
     }
     // the change of a cell since the visit began
-    __device__ __forceinline__ Pr change(const P1 &now, double v0, int eb) const
+    __device__ __forceinline__ Pr change(const P1 &now, double v0) const { return pair_of(now - split_f64(v0)); }
+    // kappa of a grid: a quarter of the parent's, whose h is half of its own
+    __device__ __forceinline__ Kap kap_of(const VisitLevel &L) const
     {
-        return pair_of(now - split_f64(v0, eb));
+        const float s = pow2f(-2 * L.id);
+        return Kap{S.kap.k3h * s, S.kap.k3l * s, S.kap.kh * s, S.kap.kl * s};
     }
 
     // ---- a box's ghosts: v0(g) + w^m (v(a) - v0(a)), a the nearest interior cell, m axes outside
@@ -273,18 +279,11 @@ struct Visit {
         return g;
     }
     __device__ __forceinline__ Pr weight(const VisitLevel &L, int m) const { return Pr{L.w[m - 1][0], L.w[m - 1][1]}; }
-    struct GhostBase {
-        double g, a;   // v0 of the ghost and of its cell
-    };
-    __device__ __forceinline__ GhostBase ghost_base(const VisitLevel &L, const Own &o, const Ghost &g) const
-    {
-        return GhostBase{v0_at(L, o.i0 + g.p, g.j, g.k), v0_at(L, o.i0 + g.pa, g.ja, g.ka)};
-    }
     // The ghosts after a half-sweep (k_patch_half's order): after the red one every ghost of the
     // sweep's result, after the black one those of the black cells.  a0, a1: the arrays of the two
-    // colours' values; d0, d1: of the ghosts.  first: the bases of ghost number tid.
+    // colours' values; d0, d1: of the ghosts.  (v0 does not change any more: it may come from L1.)
     __device__ __forceinline__ void ghosts_follow(const VisitLevel &L, const Own &o, bool black, int a0, int a1,
-                                                  int d0, int d1, const GhostBase &first, int eb)
+                                                  int d0, int d1)
     {
         const int n = ghost_count(L, o);
 #pragma unroll 1
@@ -292,53 +291,52 @@ struct Visit {
             const Ghost g = ghost(L, o, t);
             if (black && g.ca == 0)
                 continue;
-            const GhostBase v0 = t == tid ? first : ghost_base(L, o, g);
+            const double vg = MG5_AT(L.v0, vcell(L, o.i0 + g.p, g.j, g.k)),
+                         va = MG5_AT(L.v0, vcell(L, o.i0 + g.pa, g.ja, g.ka));
             const P1 now = ld(array(L, g.ca ? a1 : a0)[at(L, g.pa, g.ja, g.ka)]);
-            const P1 x = add_change(split_f64(v0.g, eb), mul_pair(weight(L, g.m), change(now, v0.a, eb)));
+            const P1 x = add_change(split_f64(vg), mul_pair(weight(L, g.m), change(now, va)));
             array(L, (g.ca ^ (g.m & 1)) ? d1 : d0)[at(L, g.p, g.j, g.k)] = st(x);
         }
     }
 
-    // Level l from its parent's residual (the top one: from the caller's v), split; c = 0.
-    __device__ __forceinline__ void enter(const VisitLevel &L, int margin)
+    // The top grid from the caller's v and f; its exponent is the whole visit's (means and ghosts of
+    // the grids below are no larger, nor are their corrections).
+    __device__ __forceinline__ void enter_top(const VisitLevel &L, int margin)
     {
         const Own o = own(L, rank);
         if (tid == 0)
             S.emax = 0;
         __syncthreads();
-        int emax = 0;
-        const VisitLevel *U = L.id > 0 ? &A.lev[L.id - 1] : nullptr;
-        const int ebu = U ? S.st[U->id].eb : 0;
         const int grow = L.nmax2 + L.Hq - 4;   // log2 of a correction's size over its residual's
-        cells(L, o, [&](int p, int j, int k) {
-            const int i = o.i0 + p;
-            double x;
-            if (U) {
-                double s = 0.0;
-                Pr r{0.0f, 0.0f};
+        const int n = o.np * L.n1 * L.n2;
+        int emax = 0;
+        double x[kHold], f[kHold];   // the first kHold cells stay in registers
+        const auto load = [&](int t, double &v, double &r) {
+            const int q = div_by(t, L.m2), k = t - q * L.n2, p = div_by(q, L.m1), j = q - p * L.n1;
+            v = v0_at(L, o.i0 + p, j, k);
+            r = MG5_AT(L.f, gcell(L, o.i0 + p, j, k));
+        };
+        const auto see = [&](double v, double r) {
+            const int ef = (__double2hiint(r) >> 20) & 0x7ff, ev = (__double2hiint(v) >> 20) & 0x7ff;
+            emax = max(emax, max(ev, ef > 0 ? min(ef + grow, 2046) : 0));
+        };
 #pragma unroll
-                for (int ch = 0; ch < 8; ++ch) {
-                    const int fi = 2 * i + (ch >> 2), fj = 2 * j + ((ch >> 1) & 1), fk = 2 * k + (ch & 1);
-                    s += __ldcg(&MG5_AT(U->v, vcell(*U, fi, fj, fk)));
-                    const float2 q = __ldcg(&MG5_AT(U->x, gcell(*U, fi, fj, fk)));
-                    r = add_pair(r, Pr{q.x, q.y});
-                }
-                x = 0.125 * s;
-                MG5_AT(L.v0, vcell(L, i, j, k)) = x;
-                Fat(L, p, j, k) = make_float2(0.125f * r.h, 0.125f * r.l);
-                // r is in units of the parent's u / h^2
-                const int er = (int)((__float_as_uint(r.h) >> 23) & 0xffu);
-                if (er > 0)
-                    emax = max(emax, min(er - 127 - 3 + ebu - kUnitBias + 1023 - U->Hq + grow, 2046));
-            } else {
-                x = v0_at(L, i, j, k);
-                const int ef = (__double2hiint(MG5_AT(L.f, gcell(L, i, j, k))) >> 20) & 0x7ff;
-                if (ef > 0)
-                    emax = max(emax, min(ef + grow, 2046));
-            }
-            emax = max(emax, (__double2hiint(x) >> 20) & 0x7ff);
-        });
+        for (int m = 0; m < kHold; ++m) {
+            x[m] = f[m] = 0.0;
+            if (tid + m * VT < n)
+                load(tid + m * VT, x[m], f[m]);
+        }
+#pragma unroll
+        for (int m = 0; m < kHold; ++m)
+            see(x[m], f[m]);
+#pragma unroll 1
+        for (int t = tid + kHold * VT; t < n; t += VT) {
+            double v, r;
+            load(t, v, r);
+            see(v, r);
+        }
         const int ng = ghost_count(L, o);
+#pragma unroll 1
         for (int t = tid; t < ng; t += VT) {   // the ghosts' fixed values
             const Ghost g = ghost(L, o, t);
             emax = max(emax, (__double2hiint(v0_at(L, o.i0 + g.p, g.j, g.k)) >> 20) & 0x7ff);
@@ -347,37 +345,74 @@ struct Visit {
         if ((tid & 31) == 0)
             atomicMax(&S.emax, emax);
         __syncthreads();
-        if (!L.single) {
-            if (tid < kVisitCtas)
-                cluster.map_shared_rank(S.ebs, tid)[rank] = S.emax;
-            cluster.sync();
-            emax = 0;
-            for (int r = 0; r < kVisitCtas; ++r)
-                emax = max(emax, S.ebs[r]);
-        } else {
-            emax = S.emax;
-        }
-        const int eb = min(max((emax == 0 ? 1023 : emax) + margin, 200), 1800);
+        // every CTA takes part, also where CTA 0 holds the grid alone
+        if (tid < kVisitCtas)
+            cluster.map_shared_rank(S.ebs, tid)[rank] = S.emax;
+        cluster.sync();
+        emax = 0;
+        for (int r = 0; r < kVisitCtas; ++r)
+            emax = max(emax, S.ebs[r]);
+        eb = min(max((emax == 0 ? 1023 : emax) + margin, 200), 1800);
         if (tid == 0) {
             // (one thread: an FP64 instruction of every warp would take 256 clocks)
-            LevelState &st = S.st[L.id];
-            st.eb = eb;
-            st.c = Pr{0.0f, 0.0f};
             const double k1 = L.k * pow2d(eb - kUnitBias), k3 = 3.0 * k1;
-            st.kap.k3h = (float)k3;
-            st.kap.k3l = (float)(k3 - (double)st.kap.k3h);
-            st.kap.kh = (float)k1;
-            st.kap.kl = (float)(k1 - (double)st.kap.kh);
+            S.kap.k3h = (float)k3;
+            S.kap.k3l = (float)(k3 - (double)S.kap.k3h);
+            S.kap.kh = (float)k1;
+            S.kap.kl = (float)(k1 - (double)S.kap.kh);
         }
+        const auto keep = [&](int t, double v, double r) {
+            const int q = div_by(t, L.m2), k = t - q * L.n2, p = div_by(q, L.m1), j = q - p * L.n1;
+            put(L, o, arr((o.i0 + p + j + k) & 1, 0), p, j, k, split_f64(v));
+            const Pr F = in_units(L, r);
+            Fat(L, p, j, k) = make_float2(F.h, F.l);
+        };
+#pragma unroll
+        for (int m = 0; m < kHold; ++m)
+            if (tid + m * VT < n)
+                keep(tid + m * VT, x[m], f[m]);
+#pragma unroll 1
+        for (int t = tid + kHold * VT; t < n; t += VT) {
+            double v, r;
+            load(t, v, r);
+            keep(t, v, r);
+        }
+    }
+    // A grid below from its parent's values and residuals, 8-child means; r comes in the parent's unit
+    // u / h^2, a quarter of its own.
+    __device__ __forceinline__ void enter_below(const VisitLevel &L, const VisitLevel &U)
+    {
+        const Own o = own(L, rank);
         cells(L, o, [&](int p, int j, int k) {
             const int i = o.i0 + p;
-            put(L, o, arr((i + j + k) & 1, 0), p, j, k, split_f64(v0_at(L, i, j, k), eb));
+            double s[8];
+            float2 q[8];
+#pragma unroll
+            for (int ch = 0; ch < 8; ++ch) {
+                const int fi = 2 * i + (ch >> 2), fj = 2 * j + ((ch >> 1) & 1), fk = 2 * k + (ch & 1);
+                s[ch] = __ldcg(&MG5_AT(U.v, vcell(U, fi, fj, fk)));
+                q[ch] = __ldcg(&MG5_AT(U.x, gcell(U, fi, fj, fk)));
+            }
+            const double x = 0.125 * (((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7])));
+            MG5_AT(L.v0, vcell(L, i, j, k)) = x;
+            const auto add2 = [&](int a) { return add_pair(Pr{q[a].x, q[a].y}, Pr{q[a + 1].x, q[a + 1].y}); };
+            const Pr r = add_pair(add_pair(add2(0), add2(2)), add_pair(add2(4), add2(6)));
+            Fat(L, p, j, k) = make_float2(0.5f * r.h, 0.5f * r.l);
+            put(L, o, arr((i + j + k) & 1, 0), p, j, k, split_f64(x));
         });
+    }
+    // ... then the ghosts' fixed values and c = 0
+    __device__ __forceinline__ void entered(const VisitLevel &L)
+    {
+        const Own o = own(L, rank);
+        const int ng = ghost_count(L, o);
+#pragma unroll 1
         for (int t = tid; t < ng; t += VT) {
             const Ghost g = ghost(L, o, t);
-            array(L, arr(g.ca ^ (g.m & 1), 0))[at(L, g.p, g.j, g.k)] =
-                st(split_f64(v0_at(L, o.i0 + g.p, g.j, g.k), eb));
+            array(L, arr(g.ca ^ (g.m & 1), 0))[at(L, g.p, g.j, g.k)] = st(split_f64(v0_at(L, o.i0 + g.p, g.j, g.k)));
         }
+        if (tid == 0)
+            S.c[L.id] = Pr{0.0f, 0.0f};
         bar(L);
     }
 
@@ -387,29 +422,27 @@ struct Visit {
     __device__ __forceinline__ void residuals(const VisitLevel &L, int mode, int b, const Pr &Pm, Pr &sum, Pr &sq)
     {
         const Own o = own(L, rank);
-        const LevelState st = S.st[L.id];
-        const VisitLevel *U = L.id > 0 ? &A.lev[L.id - 1] : nullptr;
-        // from the parent's unit u / h^2: its h is half of L's
-        const float su = U ? 4.0f * pow2f(S.st[L.id - 1].eb - st.eb) : 0.0f;
+        const Kap kap = kap_of(L);
+        const Pr c = S.c[L.id];
         Pr mean{0.0f, 0.0f};
-        if (!BOX && mode == RHS)
-            mean = U ? scale(Pm, su) : in_units(L, *A.m_up, st.eb);
-        sum = sq = Pr{0.0f, 0.0f};
+        if (!BOX && mode == RHS)   // (the parent's unit u / h^2 is four of L's)
+            mean = L.id > 0 ? scale(Pm, 4.0f) : in_units(L, *A.m_up);
+        sum = Pr{0.0f, 0.0f};
+        sq = Pr{0.0f, 0.0f};
         cells(L, o, [&](int p, int j, int k) {
             const int i = o.i0 + p, col = (i + j + k) & 1;
             Pr F;
             double v0 = 0.0;
             if (mode == RHS) {
-                const Pr g = U ? scale(Fget(L, p, j, k), su) : in_units(L, MG5_AT(L.f, gcell(L, i, j, k)), st.eb);
-                F = add_pair(mean, neg(g));
+                F = add_pair(mean, neg(Fget(L, p, j, k)));
             } else {
                 F = Fget(L, p, j, k);
                 if (mode == DOWN) {
                     v0 = v0_at(L, i, j, k);
-                    F = add_pair(F, st.c);
+                    F = add_pair(F, c);
                 }
             }
-            const Pr r = resid(lin_at(L, arr(col, b), arr(col ^ 1, b), p, j, k), F, st.kap);
+            const Pr r = resid(lin_at(L, arr(col, b), arr(col ^ 1, b), p, j, k), F, kap);
             if (mode == RHS) {
                 Fat(L, p, j, k) = make_float2(-r.h, -r.l);
                 return;
@@ -417,7 +450,7 @@ struct Visit {
             if (mode == DOWN) {
                 MG5_AT(L.x, gcell(L, i, j, k)) = make_float2(r.h, r.l);
                 // v = v0 + the change since then
-                MG5_AT(L.v, vcell(L, i, j, k)) = v0 + to_f64(change(centre(L, b, p, j, k, col), v0, st.eb), st.eb);
+                MG5_AT(L.v, vcell(L, i, j, k)) = v0 + to_f64(change(centre(L, b, p, j, k, col), v0), eb);
             } else {
                 sq = add_pair(sq, sqr(r));
             }
@@ -425,43 +458,45 @@ struct Visit {
         });
     }
 
-    // One half-sweep: the cells of `colour` from array ac (faces from ao) into array ad.
-    __device__ __forceinline__ void half(const VisitLevel &L, const Own &o, int colour, int ac, int ao, int ad,
-                                         const Pr &c, const Kap &kap)
-    {
-        const int nq = (L.n2 + 1) >> 1, n = o.np * L.n1 * nq;
-#pragma unroll 1
-        for (int t = tid; t < n; t += VT) {
-            const int g = div_by(t, L.mq), q = t - g * nq, p = div_by(g, L.m1), j = g - p * L.n1;
-            const int k = 2 * q + ((o.i0 + p + j + colour) & 1);
-            if (k >= L.n2)
-                continue;
-            const Lin1 s = lin_at(L, ac, ao, p, j, k);
-            const Pr r = resid(s, add_pair(Fget(L, p, j, k), c), kap);
-            const Pr d = neg(mul_pair(root_change(s, r, kap, clamps), Pr{L.wh, L.wl}));
-            const P1 x = add_change(ld(array(L, ac)[at(L, p, j, k)]), d);
-            if (fabsf(x.h) > kPieceMax || fabsf(d.h) > 2.0f * kPieceMax)
-                S.flag = 1;
-            put(L, o, ad, p, j, k, x);
-        }
-    }
-    // `count` sweeps after b (mod 3); returns b + count (mod 3)
+    // `count` sweeps after b (mod 3); returns b + count (mod 3).  Where a thread's cells lie (plane,
+    // row, k >> 1) is found once per call, for the first two.
     __device__ __forceinline__ int sweep(const VisitLevel &L, int count, int b)
     {
         const Own o = own(L, rank);
-        const LevelState st = S.st[L.id];
-        GhostBase first{0.0, 0.0};
-        if (tid < ghost_count(L, o))
-            first = ghost_base(L, o, ghost(L, o, tid));
+        const Kap kap = kap_of(L);
+        const Pr c = S.c[L.id];
+        const int nq = (L.n2 + 1) >> 1, n = o.np * L.n1 * nq;
+        const auto find = [&](int t) {
+            const int g = div_by(t, L.mq), p = div_by(g, L.m1);
+            return (p << 20) | ((g - p * L.n1) << 10) | (t - g * nq);
+        };
+        const int pos0 = find(tid), pos1 = find(tid + VT);
 #pragma unroll 1
         for (int s = 0; s < 2 * count; ++s) {
             const int black = s & 1, a0 = arr(0, b), a1 = arr(1, b), free_ = mod3(5 - b);
             // red: array a0 -> the free one; black: a1 -> what was a0
-            half(L, o, black, black ? a1 : a0, black ? free_ : a1, black ? a0 : free_, st.c, st.kap);
+            const int ac = black ? a1 : a0, ao = black ? free_ : a1, ad = black ? a0 : free_;
+#pragma unroll 1
+            for (int t = tid; t < n; t += VT) {
+                const int pos = t == tid ? pos0 : (t == tid + VT ? pos1 : find(t));
+                const int p = pos >> 20, j = (pos >> 10) & 1023;
+                const int k = 2 * (pos & 1023) + ((o.i0 + p + j + black) & 1);
+                if (k >= L.n2)
+                    continue;
+                const Pr F = Fget(L, p, j, k);
+                const P1 now = ld(array(L, ac)[at(L, p, j, k)]);
+                const Lin1 lin = lin_at(L, ac, ao, p, j, k);
+                const Pr r = resid(lin, add_pair(F, c), kap);
+                const Pr d = neg(mul_pair(root_change(lin, r, kap, clamps), Pr{L.wh, L.wl}));
+                const P1 x = add_change(now, d);
+                if (fabsf(x.h) > kPieceMax || fabsf(d.h) > 2.0f * kPieceMax)
+                    S.flag = 1;
+                put(L, o, ad, p, j, k, x);
+            }
             bar(L);
             if (BOX) {
                 // red: the result's arrays are free_ (red) and a0 (black); black values still in a1
-                ghosts_follow(L, o, black, free_, black ? a0 : a1, free_, a0, first, st.eb);
+                ghosts_follow(L, o, black, free_, black ? a0 : a1, free_, a0);
                 __syncthreads();
             }
             if (black)
@@ -477,26 +512,21 @@ struct Visit {
             x = add_pair(x, shfl_down(x, q));
             y = add_pair(y, shfl_down(y, q));
         }
+        turn ^= 1;   // (the other buffer's readers have passed a barrier since)
         if ((tid & 31) == 0) {
-            S.red[0][tid >> 5] = x;
-            S.red[1][tid >> 5] = y;
+            S.red[turn][0][tid >> 5] = x;
+            S.red[turn][1][tid >> 5] = y;
         }
         __syncthreads();
-        if (tid < 32) {
-            x = tid < VT / 32 ? S.red[0][tid] : Pr{0.0f, 0.0f};
-            y = tid < VT / 32 ? S.red[1][tid] : Pr{0.0f, 0.0f};
-            for (int q = VT / 64; q > 0; q >>= 1) {
-                x = add_pair(x, shfl_down(x, q));
-                y = add_pair(y, shfl_down(y, q));
-            }
-            if (tid == 0) {
-                S.bc[0] = x;
-                S.bc[1] = y;
-            }
+        x = S.red[turn][0][tid & 15];
+        y = S.red[turn][1][tid & 15];
+        const auto other = [](const Pr &z, int q) {
+            return Pr{__shfl_xor_sync(0xffffffffu, z.h, q), __shfl_xor_sync(0xffffffffu, z.l, q)};
+        };
+        for (int q = VT / 64; q > 0; q >>= 1) {
+            x = add_pair(x, other(x, q));
+            y = add_pair(y, other(y, q));
         }
-        __syncthreads();
-        x = S.bc[0];
-        y = S.bc[1];
     }
     // After the DOWN residuals: the mean residual (periodic), taken off c.
     __device__ __forceinline__ Pr mean_residual(const VisitLevel &L, Pr sum)
@@ -517,7 +547,7 @@ struct Visit {
         }
         mean = mul_pair(sum, Pr{L.inv_h, L.inv_l});
         if (tid == 0)
-            S.st[L.id].c = add_pair(S.st[L.id].c, neg(mean));
+            S.c[L.id] = add_pair(S.c[L.id], neg(mean));
         __syncthreads();
         return mean;
     }
@@ -525,10 +555,9 @@ struct Visit {
     __device__ __forceinline__ void leave_up(const VisitLevel &L, int b)
     {
         const Own o = own(L, rank);
-        const int eb = S.st[L.id].eb;
         cells(L, o, [&](int p, int j, int k) {
             const int i = o.i0 + p;
-            const Pr e = change(centre(L, b, p, j, k, (i + j + k) & 1), v0_at(L, i, j, k), eb);
+            const Pr e = change(centre(L, b, p, j, k, (i + j + k) & 1), v0_at(L, i, j, k));
             MG5_AT(L.x, vcell(L, i, j, k)) = make_float2(e.h, e.l);
         });
         const int ng = ghost_count(L, o);
@@ -537,7 +566,7 @@ struct Visit {
             const int i = o.i0 + g.p;
             if (i >= 0 && i < L.n0 && (g.p < 0 || g.p >= o.np))
                 continue;   // a neighbour's plane
-            const Pr e = change(centre(L, b, g.pa, g.ja, g.ka, g.ca), v0_at(L, o.i0 + g.pa, g.ja, g.ka), eb);
+            const Pr e = change(centre(L, b, g.pa, g.ja, g.ka, g.ca), v0_at(L, o.i0 + g.pa, g.ja, g.ka));
             const Pr w = mul_pair(weight(L, g.m), e);
             MG5_AT(L.x, vcell(L, i, g.j, g.k)) = make_float2(w.h, w.l);
         }
@@ -547,8 +576,6 @@ struct Visit {
     {
         const Own o = own(L, rank);
         const VisitLevel &D = A.lev[L.id + 1];
-        const int eb = S.st[L.id].eb, ebd = S.st[D.id].eb;
-        const float s64 = pow2f(ebd - eb) * (1.0f / 64.0f);
         const auto three = [](const Pr &x, const Pr &y) {   // 3 x + y
             const float p = mul(3.0f, x.h), e = fma(3.0f, x.h, -p);
             const Pr s = two_sum(p, y.h);
@@ -569,7 +596,7 @@ struct Visit {
             };
             const auto line = [&](int x, int y) { return three(E(x, y, a[2]), E(x, y, n[2])); };
             const Pr y0 = three(line(a[0], a[1]), line(a[0], n[1])), y1 = three(line(n[0], a[1]), line(n[0], n[1]));
-            const Pr d = scale(three(y0, y1), s64);
+            const Pr d = scale(three(y0, y1), 1.0f / 64.0f);
             const P1 x = add_change(centre(L, b, p, j, k, col), d);
             if (fabsf(x.h) > kPieceMax || fabsf(d.h) > 2.0f * kPieceMax)
                 S.flag = 1;
@@ -577,10 +604,10 @@ struct Visit {
         });
         if (!BOX) {
             // c of the grid below from its unit u / h^2 (h^2 four times this one's)
-            const Pr c = add_pair(S.st[L.id].c, scale(S.st[D.id].c, 0.25f * pow2f(ebd - eb)));
+            const Pr c = add_pair(S.c[L.id], scale(S.c[D.id], 0.25f));
             __syncthreads();
             if (tid == 0)
-                S.st[L.id].c = c;
+                S.c[L.id] = c;
         }
         bar(L);
     }
@@ -593,7 +620,7 @@ struct Visit {
             const Pr m = mul_pair(sum, Pr{L.inv_h, L.inv_l});
             sq = add_pair(sq, neg(mul_pair(sum, m)));
             if (tid == 0)
-                S.st[L.id].c = neg(m);
+                S.c[L.id] = neg(m);
             __syncthreads();
         }
         const float rn = sq.h > 0.0f ? sq.h : 0.0f;
@@ -618,6 +645,7 @@ struct Visit {
         int l = 0, b = 0, it = 0, step = ENTER;
         float r0 = -1.0f;
         Pr mean{0.0f, 0.0f};
+        enter_top(A.lev[0], margin);
         if (split_at == 0 && rank != 0)
             step = DONE;
 #pragma unroll 1
@@ -626,17 +654,20 @@ struct Visit {
             int count = 0;
             if (step == UPWARD) {
                 if (l == split_at - 1) {
-                    // CTA 0's correction, with its unit and c, for the grid that the CTAs share
-                    if (rank == 0 && tid > 0 && tid < kVisitCtas)
-                        cluster.map_shared_rank(S.st, tid)[split_at] = S.st[split_at];
+                    // CTA 0's correction, with its c, for the grid that the CTAs share
+                    if (!BOX && rank == 0 && tid > 0 && tid < kVisitCtas)
+                        cluster.map_shared_rank(S.c, tid)[split_at] = S.c[split_at];
                     cluster.sync();
                 }
                 prolong(L, bdn);
                 b = bdn;
                 count = A.nu2;
             } else {
-                if (step == ENTER)
-                    enter(L, margin);
+                if (step == ENTER) {
+                    if (l > 0)
+                        enter_below(L, A.lev[l - 1]);
+                    entered(L);
+                }
                 Pr sum, sq;
                 residuals(L, step == ENTER ? RHS : (step == DOWNWARD ? DOWN : TEST), step == ENTER ? 0 : b, mean, sum,
                           sq);
@@ -697,25 +728,36 @@ struct Visit {
         // the top grid's iterate and c
         const VisitLevel &L = A.lev[0];
         const Own o = own(L, rank);
-        const LevelState st = S.st[0];
-        cells(L, o, [&](int p, int j, int k) {
-            const int i = o.i0 + p;
-            const double v0 = v0_at(L, i, j, k);
-            MG5_AT(L.v, vcell(L, i, j, k)) =
-                v0 + to_f64(change(centre(L, b, p, j, k, (i + j + k) & 1), v0, st.eb), st.eb);
-        });
+        const int n = o.np * L.n1 * L.n2;
+#pragma unroll 1
+        for (int t0 = tid; t0 < n; t0 += kHold * VT) {
+            double v0[kHold];
+#pragma unroll
+            for (int m = 0; m < kHold; ++m) {
+                const int t = t0 + m * VT, q = div_by(t, L.m2), k = t - q * L.n2, p = div_by(q, L.m1), j = q - p * L.n1;
+                v0[m] = t < n ? v0_at(L, o.i0 + p, j, k) : 0.0;
+            }
+#pragma unroll
+            for (int m = 0; m < kHold; ++m) {
+                const int t = t0 + m * VT, q = div_by(t, L.m2), k = t - q * L.n2, p = div_by(q, L.m1), j = q - p * L.n1;
+                const int i = o.i0 + p;
+                if (t < n)
+                    MG5_AT(L.v, vcell(L, i, j, k)) =
+                        v0[m] + to_f64(change(centre(L, b, p, j, k, (i + j + k) & 1), v0[m]), eb);
+            }
+        }
         const int ng = ghost_count(L, o);
         for (int t = tid; t < ng; t += VT) {
             const Ghost g = ghost(L, o, t);
             const int i = o.i0 + g.p;
             if (i >= 0 && i < L.n0 && (g.p < 0 || g.p >= o.np))
                 continue;
-            const GhostBase v0 = ghost_base(L, o, g);
-            const Pr e = change(centre(L, b, g.pa, g.ja, g.ka, g.ca), v0.a, st.eb);
-            MG5_AT(L.v, vcell(L, i, g.j, g.k)) = v0.g + to_f64(mul_pair(weight(L, g.m), e), st.eb);
+            const Pr e = change(centre(L, b, g.pa, g.ja, g.ka, g.ca), v0_at(L, o.i0 + g.pa, g.ja, g.ka));
+            MG5_AT(L.v, vcell(L, i, g.j, g.k)) =
+                v0_at(L, i, g.j, g.k) + to_f64(mul_pair(weight(L, g.m), e), eb);
         }
         if (!BOX && rank == 0 && tid == 0)
-            *A.c_out = to_f64(st.c, st.eb) / L.h2;
+            *A.c_out = to_f64(S.c[0], eb) / L.h2;
         return true;
     }
 };

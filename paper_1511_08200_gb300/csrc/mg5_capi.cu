@@ -651,10 +651,10 @@ struct Run64 {
     }
 
     // The visit of grid l and every grid below it in one launch (k_visit.cu); false: not these grids.
-    // Sides up to 32: a 64^3 grid's planes do not fit 16 SMs, and its launches fill the GPU.
     bool visit(int l, cudaError_t *e)
     {
-        if (h->n[l] > 32 || h->n[h->nlev - 1] >= kSpectralMinSide)
+        const int n = h->n[l];
+        if ((long long)n * n * n > kVisitCells || h->n[h->nlev - 1] >= kSpectralMinSide)
             return false;
         VisitArgs A = {};
         int q[kMaxLevels][3];

@@ -6,7 +6,10 @@ namespace mg5 {
 
 constexpr int kVisitCtas = 16;
 constexpr int kVisitLevels = 6;
-constexpr int kVisitCells = 40 * 32 * 32;    // cells of the largest patch grid taken
+// Cells of the largest grid taken.  A half-sweep of 32^3 costs 16 SMs 4.9 us (450 instructions a cell)
+// where a launch over all SMs takes 3.1 us (patch 5.2): a 64^3 refinement took 1497 us with the 32^3
+// grid in the cluster and 1423 without; 24 x 20 x 36 (2.2 us a half-sweep) gained 5% in it.
+constexpr int kVisitCells = 20000;
 constexpr int kVisitCoarsest = 2048;          // cells of a coarsest grid CTA 0 iterates
 constexpr int kVisitSmem = 222 * 1024;        // dynamic shared memory a CTA may use
 
