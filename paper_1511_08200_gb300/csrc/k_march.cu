@@ -30,7 +30,9 @@
 // The plane values, sums and differences of e and B travel as (e, B) pairs through the
 // packed FP32 instructions (two lanes an instruction).  Every cell is updated by the same
 // arithmetic on the same operands, in the same order, as the gather-based kernels
-// (parts2_of, cell_update_corr_parts), so the result is the same sweep to the bit.  Periodic in i, j, k; n a multiple of 32; out of place.
+// (parts2_of, cell_update_corr_parts), so the result is the same sweep to the bit.  Periodic in i, j, k; n a multiple of 4 (rows come
+// in 16-byte copies); out of place.  Against the gather-based fused kernel: 64^3 10.4 -> 6.3 us,
+// 120^3 28.3 -> 17.7, 240^3 128 -> 105, 512^3 1117 -> 795.
 #include <type_traits>
 
 #include "mg5_async.cuh"
@@ -194,6 +196,11 @@ __global__ void __launch_bounds__(MT_THREADS, 2)
     const bool a_even = ((q0 + 1 + jA + kA) & 1) == 0;   // A active on steps q0, q0 + 2, ...
     const Pos pos[2] = {a_even ? pA : pB, a_even ? pB : pA};
     const bool first[2] = {a_even, !a_even};   // tile pairs: A is the pair's first cell
+    // in the last tiles of a side that is not a multiple of 16 and 32, the positions past the side
+    // are the periodic images of positions 0, 1, ...: those at the side itself give the last row and
+    // column their new red faces, the rest have no work, and none is written
+    const bool act = (tile || ring) && jA <= n && kA <= n;
+    const bool own = tile && jA < n && kA < n;
     float *optr = out + (long long)i0 * n2 + (long long)(tile ? jA : j0) * n + (tile ? kA : k0);
     ColCache cc[2] = {};
     float rprev = 0.0f;   // red value of the step before (its plane's red cell)
@@ -205,7 +212,7 @@ __global__ void __launch_bounds__(MT_THREADS, 2)
     auto step = [&](auto S0c, auto SETc, bool warm) {
         constexpr int s0 = decltype(S0c)::value, set = decltype(SETc)::value;
         constexpr int s1 = (s0 + 1) % MNS, s2 = (s0 + 2) % MNS;
-        if (tile || ring) {
+        if (act) {
             ColCache &c = cc[set];
             const Pos ps = pos[set];
             const float *E0 = E + s0 * MPL + ps.off, *E1 = E + s1 * MPL + ps.off,
@@ -229,7 +236,7 @@ __global__ void __launch_bounds__(MT_THREADS, 2)
                                                     cf, clamped);
             MG5_AT(S.RN[(set + 1) & 1], ps.rn) = r1;   // plane p + 1 (p - i0 has the parity of set)
             const float2 rB1 = make_float2(r1, q1.c.y);
-            if (tile && !warm) {
+            if (own && !warm) {
                 // black cell (p) of the position: new red faces, old edges
                 const float *rn = S.RN[set & 1] + ps.rn;
                 const float sye = __fadd_rn(MG5_AT(rn, RNO), MG5_AT(rn, -RNO)), sze = __fadd_rn(MG5_AT(rn, 1), MG5_AT(rn, -1));
@@ -347,27 +354,44 @@ __global__ void __launch_bounds__(MT_THREADS, 2)
 
 bool march_ok(int n) { return n >= MT_K && n % MT_K == 0 && n % MT_J == 0; }
 
+// Sides that the tiles do not divide: the positions past the side in the last tiles are work for
+// nothing (a third of all at 48), and the march is still faster than the fused kernel at every side
+// that its 16-byte copies can read (the best chunk of the fused kernel -> march: 36^3 10.0 -> 5.7 us,
+// 48^3 10.5 -> 5.5, 72^3 10.8 -> 8.5, 120^3 28 -> 17.7, 176^3 58 -> 45.6, 240^3 128 -> 104).
+bool march_ragged_ok(int n) { return n > MT_K && n % 4 == 0; }
+
 cudaError_t launch_sweep_march(const float *in, float *out, const float *f, const float *B,
                                const double *cptr, int n, CoefT<float> cf,
                                unsigned long long *clamp, cudaStream_t st, int chunk)
 {
-    if (!march_ok(n) || !B)
+    if (!(march_ok(n) || march_ragged_ok(n)) || !B)
         return cudaErrorInvalidValue;
-    const int tiles = (n / MT_K) * (n / MT_J);
+    const int tk = (n + MT_K - 1) / MT_K, tj = (n + MT_J - 1) / MT_J, tiles = tk * tj;
     int ichunk = chunk;
     if (ichunk <= 0) {
-        // about six waves of two CTAs per SM over 152 SMs, chunks of at least 16 planes
-        int chunks = (6 * 2 * 152 + tiles - 1) / tiles;
-        if (chunks > n / 16)
-            chunks = n / 16;
-        if (chunks < 1)
-            chunks = 1;
-        ichunk = (n + chunks - 1) / chunks;
+        if (tiles * (n / 16) >= 2 * 152) {
+            // about six waves of two CTAs per SM over 152 SMs, chunks of at least 16 planes
+            int chunks = (6 * 2 * 152 + tiles - 1) / tiles;
+            if (chunks > n / 16)
+                chunks = n / 16;
+            if (chunks < 1)
+                chunks = 1;
+            ichunk = (n + chunks - 1) / chunks;
+        } else {
+            // fewer CTAs than the GPU holds: the sweep takes as long as one CTA, a chunk's planes
+            // and the two before it one after the other, so the shortest chunk that fits at once (64^3:
+            // 12.4 us with chunks of 16 planes, 6.3 with 4).  Not below 4 planes: of shorter chunks
+            // half the work is the two extra planes, and boxes that share the GPU pay for it (a batch
+            // of 24 boxes of 32^3 .. 128^3: 13.9 ms with 16 planes, 13.6 with 4, 14.3 with 2)
+            ichunk = 4;
+            while (tiles * ((n + ichunk - 1) / ichunk) > 2 * 152)
+                ++ichunk;
+        }
     }
     if (ichunk > n)
         ichunk = n;
     const int chunks = (n + ichunk - 1) / ichunk;
-    dim3 grid(n / MT_K, n / MT_J, chunks);
+    dim3 grid(tk, tj, chunks);
     k_sweep_march<<<grid, MT_THREADS, sizeof(MarchSmem), st>>>(in, out, f, B, cptr, n, ichunk, cf,
                                                               clamp);
     count_launch(1);

@@ -128,8 +128,9 @@ inline bool fused_ok(int n)
 }
 cudaError_t prepare_fused_kernels();
 // FP32 correction-form sweep as a column march (k_march.cu): 16 x 32 tiles, n a multiple
-// of 32, B required; `chunk` planes per CTA (0: about six waves of two CTAs per SM)
+// of 32, B required; `chunk` planes per CTA (0: chosen by the number of tiles)
 bool march_ok(int n);
+bool march_ragged_ok(int n);   // other sides whose last tiles it can run part-filled
 cudaError_t launch_sweep_march(const float *in, float *out, const float *f, const float *B,
                                const double *cptr, int n, CoefT<float> cf,
                                unsigned long long *clamp, cudaStream_t st, int chunk = 0);
@@ -137,7 +138,8 @@ cudaError_t prepare_march_kernel();
 
 // How one grid side is swept (speed only: every schedule computes the same values).
 struct SweepSchedule {
-    int form = 0;     // 0: two-pass, 1: fused, 2: column march (FP32 correction form)
+    int form = 0;     // 0: two-pass, 1: fused (chunk 0, FP32: the march where it is as exact and faster),
+                      // 2: column march (FP32 correction form)
     int block = kBlock;
     int chunk = 0;
     float ms = 0.f;   // tuned time of one sweep (0: not measured)
@@ -160,8 +162,14 @@ cudaError_t launch_sweep_sched(const SweepSchedule &s, const T *in, T *out, cons
         if (s.form == 2 && B && march_ok(n))
             return launch_sweep_march(in, out, f, B, cptr, n, cf, clamp, st, s.chunk);
     }
-    if ((s.form == 1 || s.form == 2) && fused_ok<T>(n))
+    if ((s.form == 1 || s.form == 2) && fused_ok<T>(n)) {
+        // the same values as the fused kernel, faster; a set chunk of planes means that kernel
+        if constexpr (sizeof(T) == 4) {
+            if (B && !march_ok(n) && march_ragged_ok(n) && !(s.form == 1 && s.chunk))
+                return launch_sweep_march(in, out, f, B, cptr, n, cf, clamp, st, 0);
+        }
         return launch_sweep_fused<T>(in, out, f, cptr, n, cf, clamp, st, B, s.form == 1 ? s.chunk : 0);
+    }
     return launch_sweep<T>(in, out, f, cptr, n, cf, clamp, st, B, s.block);
 }
 template <typename T>

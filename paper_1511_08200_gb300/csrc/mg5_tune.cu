@@ -89,8 +89,8 @@ std::vector<SweepSchedule> candidates(int precision, int n)
     }
     const bool fused = precision == MG5_MIXED ? fused_ok<float>(n) : fused_ok<double>(n);
     if (fused)
-        for (int c : {8, 16, 32})
-            if (c <= n) {
+        for (int c : {0, 8, 16, 32})
+            if (c <= n && (c || (precision == MG5_MIXED && march_ragged_ok(n)))) {
                 SweepSchedule s;
                 s.form = 1;
                 s.chunk = c;
