@@ -7,6 +7,8 @@
 // Paper: arXiv:1511.08200, Eq. (eomvarphi), Eq. (newton), Sec. 3.1 (level
 // solve, V-cycles, boundary values from the coarser level), Sec. 3.2
 // (interpolated fine phi, force by central differences).
+#include <type_traits>
+
 #include "mg5_fin.cuh"
 
 namespace mg5 {
@@ -900,65 +902,80 @@ struct RefineSrc {
     int periodic;     // 1: wrap indices modulo c (cube)
 };
 
+// FP64 bound as a sum of eight weighted values (~40 FP64 operations a cell: 21 us for 66^3): the
+// weights are 3/4 and 1/4 of the nearer and the farther centre on each axis, so the axes go one
+// after the other as 3 near + far with the three factors 1/4 in one exact 1/64 at the end, eight
+// FP64 operations a cell.  Indices in 32 bits where the arrays have fewer than 2^31 cells
+// (a 64-bit division is ~100 instructions).
+template <typename Int>
 __global__ void k_refine(const double *__restrict__ phic, RefineSrc src, int o0, int o1, int o2,
                          int d0, int d1, int d2, int g, double *__restrict__ fine)
 {
-    const long long total = (long long)d0 * d1 * d2;
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    using UInt = typename std::make_unsigned<Int>::type;
+    const UInt total = (UInt)d0 * (UInt)d1 * (UInt)d2;
+    const UInt t = (UInt)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= total)
         return;
-    const int K = (int)(t % d2);
-    const long long q = t / d2;
-    const int J = (int)(q % d1), I = (int)(q / d1);
+    const UInt q = t / (UInt)d2;
+    const int K = (int)(t - q * (UInt)d2);
+    const int I = (int)(q / (UInt)d1), J = (int)(q - (UInt)I * (UInt)d1);
     const int loc[3] = {I, J, K};
     const int org[3] = {o0, o1, o2};
     const int dim[3] = {src.c0, src.c1, src.c2};
-    int lo[3], hi[3];
-    double w[3];
+    int at[3][2];   // stored indices of the nearer and the farther centre
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        // 4 t = 4 o + 2 (I - g) - 1 is an exact integer
+        // 4 t = 4 o + 2 (I - g) - 1 is an odd integer: a quarter (lo is nearer) or three of the way
         const int t4 = 4 * org[a] + 2 * (loc[a] - g) - 1;
-        const int i0 = (t4 >= 0) ? (t4 >> 2) : -((-t4 + 3) >> 2);
-        w[a] = (double)(t4 - 4 * i0) * 0.25;
+        const int i0 = t4 >> 2;   // floor
+        int lo, hi;
         if (src.periodic) {
             int l = i0 % dim[a];
             l = l < 0 ? l + dim[a] : l;
-            lo[a] = l;
-            hi[a] = (l + 1 == dim[a]) ? 0 : l + 1;
+            lo = l;
+            hi = (l + 1 == dim[a]) ? 0 : l + 1;
         } else {
-            lo[a] = i0 + src.pg;
-            hi[a] = i0 + 1 + src.pg;
+            lo = i0 + src.pg;
+            hi = i0 + 1 + src.pg;
         }
+        const bool quarter = (t4 & 3) == 1;
+        at[a][0] = quarter ? lo : hi;
+        at[a][1] = quarter ? hi : lo;
     }
-    const long long C1 = src.c1, C2 = src.c2;
-    double v = 0.0;
+    double y[2];
 #pragma unroll
-    for (int a = 0; a < 2; ++a)
+    for (int a = 0; a < 2; ++a) {
+        double x[2];
 #pragma unroll
-        for (int b = 0; b < 2; ++b)
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const double wt = (a ? w[0] : 1.0 - w[0]) * (b ? w[1] : 1.0 - w[1]) *
-                                  (c ? w[2] : 1.0 - w[2]);
-                const long long idx =
-                    ((long long)(a ? hi[0] : lo[0]) * C1 + (b ? hi[1] : lo[1])) * C2 +
-                    (c ? hi[2] : lo[2]);
-                v += wt * MG5_AT(phic, idx);
-            }
-    MG5_AT(fine, t) = v;
+        for (int b = 0; b < 2; ++b) {
+            const Int row = ((Int)at[0][a] * src.c1 + at[1][b]) * src.c2;
+            x[b] = fma(3.0, MG5_AT(phic, row + at[2][0]), MG5_AT(phic, row + at[2][1]));
+        }
+        y[a] = fma(3.0, x[0], x[1]);
+    }
+    MG5_AT(fine, t) = fma(3.0, y[0], y[1]) * (1.0 / 64.0);
+}
+
+static cudaError_t refine_any(const double *phic, const RefineSrc &src, const int o[3], int d0, int d1,
+                              int d2, int ghost, double *fine, cudaStream_t st)
+{
+    const long long work = (long long)d0 * d1 * d2;
+    const long long limit = (1ll << 31) - 1024;   // the last block's threads count past the end
+    if (work < limit && (long long)src.c0 * src.c1 * src.c2 < limit)
+        k_refine<int><<<grid_spread(work), block_spread(work), 0, st>>>(phic, src, o[0], o[1], o[2], d0,
+                                                                        d1, d2, ghost, fine);
+    else
+        k_refine<long long><<<grid_spread(work), block_spread(work), 0, st>>>(
+            phic, src, o[0], o[1], o[2], d0, d1, d2, ghost, fine);
+    count_launch(1);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_refine(const double *phic, int nc, const int o[3], const int pn[3], int ghost,
                           double *fine, cudaStream_t st)
 {
     const int d0 = 2 * pn[0] + 2 * ghost, d1 = 2 * pn[1] + 2 * ghost, d2 = 2 * pn[2] + 2 * ghost;
-    const long long work = (long long)d0 * d1 * d2;
-    const RefineSrc src{nc, nc, nc, 0, 1};
-    k_refine<<<grid_spread(work), block_spread(work), 0, st>>>(phic, src, o[0], o[1], o[2], d0, d1, d2, ghost,
-                                                  fine);
-    count_launch(1);
-    return cudaGetLastError();
+    return refine_any(phic, RefineSrc{nc, nc, nc, 0, 1}, o, d0, d1, d2, ghost, fine, st);
 }
 
 // Tricubic variant (periodic source): per axis the fine centre sits a quarter cell right
@@ -1021,12 +1038,7 @@ cudaError_t launch_refine_box(const double *box, const int bd[3], int pg, const 
                               const int pn[3], int ghost, double *fine, cudaStream_t st)
 {
     const int d0 = 2 * pn[0] + 2 * ghost, d1 = 2 * pn[1] + 2 * ghost, d2 = 2 * pn[2] + 2 * ghost;
-    const long long work = (long long)d0 * d1 * d2;
-    const RefineSrc src{bd[0], bd[1], bd[2], pg, 0};
-    k_refine<<<grid_spread(work), block_spread(work), 0, st>>>(box, src, o[0], o[1], o[2], d0, d1, d2, ghost,
-                                                  fine);
-    count_launch(1);
-    return cudaGetLastError();
+    return refine_any(box, RefineSrc{bd[0], bd[1], bd[2], pg, 0}, o, d0, d1, d2, ghost, fine, st);
 }
 
 // --------------------------------------------------------------------------
