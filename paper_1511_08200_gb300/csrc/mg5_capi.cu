@@ -972,6 +972,8 @@ int mg5_create(mg5_ctx **out, int device, size_t budget)
         e = prepare_fused_kernels();
     if (e == cudaSuccess)
         e = prepare_visit_kernels();
+    if (e == cudaSuccess)
+        e = prepare_bottom_kernel();
     if (e != cudaSuccess) {
         cudaGetLastError();
         mg5_destroy(ctx);
