@@ -473,102 +473,17 @@ __global__ void k_prolong_add(const T *__restrict__ vc, const T *__restrict__ v0
         }
 }
 
-// The same prolongation as a march along i (coarse sides >= 128): one thread per coarse
-// column (J, K) over a chunk of coarse planes.  The k- and j-stages of a coarse plane (Y[cj][ck] below, the values of
-// k_prolong_add's Y for that plane) are formed once when the plane enters and kept for the
-// three coarse planes that use them, so each coarse value is read and differenced once per
-// chunk instead of 27 times and each stage runs once per plane; the i-stage and the fine
-// update are k_prolong_add's, so both kernels give the same values.
-template <typename T>
-__global__ void k_prolong_march(const T *__restrict__ vc, const T *__restrict__ v0c, int nc,
-                                int ichunk, T *__restrict__ vf, double *c_fine,
-                                const double *c_coarse)
-{
-    const int K = blockIdx.x * blockDim.x + threadIdx.x;
-    const int J = blockIdx.y;
-    const int I0 = blockIdx.z * ichunk;
-    const int I1 = min(I0 + ichunk, nc);
-    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0 && c_fine &&
-        c_coarse)
-        MG5_AT(c_fine, 0) += MG5_AT(c_coarse, 0);
-    if (K >= nc)
-        return;
-    const long long NC = nc;
-    const int kk[3] = {K == 0 ? nc - 1 : K - 1, K, K == nc - 1 ? 0 : K + 1};
-    const int jj[3] = {J == 0 ? nc - 1 : J - 1, J, J == nc - 1 ? 0 : J + 1};
-    // Y[cj][ck] of coarse plane i
-    auto yplane = [&](int i, T y[2][2]) {
-        T Z[3][2];
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            const long long row = ((long long)i * NC + jj[b]) * NC;
-            T e[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c)
-                e[c] = v0c ? MG5_AT(vc, row + kk[c]) - MG5_AT(v0c, row + kk[c]) : MG5_AT(vc, row + kk[c]);
-            Z[b][0] = fma((T)3, e[1], e[0]);
-            Z[b][1] = fma((T)3, e[1], e[2]);
-        }
-#pragma unroll
-        for (int cj = 0; cj < 2; ++cj)
-#pragma unroll
-            for (int ck = 0; ck < 2; ++ck)
-                y[cj][ck] = fma((T)3, Z[1][ck], Z[cj ? 2 : 0][ck]);
-    };
-    T ym[2][2], y0[2][2], yp[2][2];   // planes I - 1, I, I + 1
-    yplane(I0 == 0 ? nc - 1 : I0 - 1, ym);
-    yplane(I0, y0);
-    const int n = 2 * nc;
-    const T w = (T)(1.0 / 64.0);
-    using V = typename Vec2<T>::type;
-    for (int I = I0; I < I1; ++I) {
-        yplane(I == nc - 1 ? 0 : I + 1, yp);
-#pragma unroll
-        for (int ci = 0; ci < 2; ++ci)
-#pragma unroll
-            for (int cj = 0; cj < 2; ++cj) {
-                const T o0 = fma((T)3, y0[cj][0], ci ? yp[cj][0] : ym[cj][0]);
-                const T o1 = fma((T)3, y0[cj][1], ci ? yp[cj][1] : ym[cj][1]);
-                const long long f = ((long long)(2 * I + ci) * n + (2 * J + cj)) * n + 2 * K;
-                V *p = &MG5_AT(reinterpret_cast<V *>(vf + f), 0);
-                V v = *p;
-                v.x = fma(o0, w, v.x);
-                v.y = fma(o1, w, v.y);
-                *p = v;
-            }
-#pragma unroll
-        for (int cj = 0; cj < 2; ++cj)
-#pragma unroll
-            for (int ck = 0; ck < 2; ++ck) {
-                ym[cj][ck] = y0[cj][ck];
-                y0[cj][ck] = yp[cj][ck];
-            }
-    }
-}
-
 template <typename T>
 cudaError_t launch_prolong_add(const T *vc, const T *v0c, int nc, T *vf, double *c_fine,
                                const double *c_coarse, cudaStream_t st)
 {
-    if (nc >= 128) {
-        // columns (J, K) x chunks of planes: about a million threads, chunks of >= 4 planes.
-        // Below 128^3 coarse cells the gather kernel's four times as many threads hide more
-        // latency than the march saves (measured: a 128^3 FP64 solve's prolongations took
-        // 0.56 ms with the march, 0.49 ms with the gather; at 512^3 the march halved them)
-        const int tx = nc < 256 ? ((nc + 31) / 32) * 32 : 256;
-        int chunks = (int)((1ll << 20) / ((long long)nc * nc));
-        if (chunks > nc / 4)
-            chunks = nc / 4;
-        if (chunks < 1)
-            chunks = 1;
-        const int ichunk = (nc + chunks - 1) / chunks;
-        chunks = (nc + ichunk - 1) / ichunk;
-        dim3 grid((nc + tx - 1) / tx, nc, chunks);
-        k_prolong_march<T><<<grid, tx, 0, st>>>(vc, v0c, nc, ichunk, vf, c_fine, c_coarse);
-    } else {
-        const long long work = (long long)nc * nc * nc;
-        k_prolong_add<T><<<grid_spread(work), block_spread(work), 0, st>>>(vc, v0c, nc, vf, c_fine, c_coarse);
-    }
+    // Above 32^3 coarse cells as tiles (72^3 fine: 10.5 -> 8.6 us in FP64, 5.5 -> 5.1 in FP32; larger
+    // grids in k_prolong.cu); below, the gather kernel's threads are enough to hide its loads and a
+    // tile's two phases cost more (56^3 fine, FP64: 6.9 us, 8.5 as tiles; 64^3: 9.0 and 8.7)
+    if (nc > 32)
+        return launch_prolong_tile<T>(vc, v0c, nc, vf, c_fine, c_coarse, st);
+    const long long work = (long long)nc * nc * nc;
+    k_prolong_add<T><<<grid_spread(work), block_spread(work), 0, st>>>(vc, v0c, nc, vf, c_fine, c_coarse);
     count_launch(1);
     return cudaGetLastError();
 }

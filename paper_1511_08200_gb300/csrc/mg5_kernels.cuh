@@ -209,6 +209,10 @@ template <typename T>
 cudaError_t launch_coarse_rhs(const T *vc, T *fc, const double *m_fine, double *c_coarse, int nc,
                               CoefT<T> cfc, cudaStream_t st, const T *B = nullptr);
 // vf += P(vc - v0c) (v0c may be NULL: plain prolongation of vc); c_fine += c_coarse if both non-NULL
+// ... as tiles (k_prolong.cu): nc > 32
+template <typename T>
+cudaError_t launch_prolong_tile(const T *vc, const T *v0c, int nc, T *vf, double *c_fine,
+                                const double *c_coarse, cudaStream_t st);
 template <typename T>
 cudaError_t launch_prolong_add(const T *vc, const T *v0c, int nc, T *vf, double *c_fine,
                                const double *c_coarse, cudaStream_t st);
