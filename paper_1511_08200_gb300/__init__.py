@@ -269,18 +269,41 @@ def workspace_bytes(n: int, precision=FP64) -> int:
     return out.value
 
 
+# A truncated level is two calls whose kernels take 12 us: the 11 us that each call spent in Python set
+# its time (24 us; a torch Stream object for its handle alone 2.9 us, module and attribute look-ups at
+# every argument).
+_DTYPES = {}
+
+
+def _torch(dtype: str):
+    """(torch, the dtype of that name), looked up once a name."""
+    got = _DTYPES.get(dtype)
+    if got is None:
+        import torch
+        got = _DTYPES[dtype] = (torch, getattr(torch, dtype))
+    return got
+
+
+def _current_stream() -> int:
+    """The handle of torch's current stream on the current device."""
+    torch = _torch("float64")[0]
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
+
+
 def _ptr(t, dtype="float64", device=None) -> int:
     """Device pointer of a contiguous torch CUDA tensor of the given dtype (on `device`
     when given), or None."""
     if t is None:
         return None
-    import torch
-    want = getattr(torch, dtype)
-    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == want and t.is_contiguous()):
+    torch, want = _torch(dtype)
+    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is want and t.is_contiguous()):
         raise TypeError("expected a contiguous %s CUDA tensor" % dtype)
-    if device is not None and (t.device.index or 0) != device:
+    if device is not None and t.get_device() != device:
         raise MG5Error(E_ARG, "tensor on cuda:%d, the context is on cuda:%d"
-                       % (t.device.index or 0, device))
+                       % (t.get_device(), device))
     if _BOUNDS:
         _lib.mg5_bounds_note(t.data_ptr())
     return t.data_ptr()
@@ -302,12 +325,12 @@ def bounds_check():
 # Shape checks, made before any pointer reaches the library: a buffer of the wrong size
 # would make the kernels read or write past its end.
 def _dims(t) -> tuple:
-    return tuple(int(x) for x in t.shape)
+    return tuple(map(int, t.shape))
 
 
 def _want(t, shape, name: str):
     """MG5Error(E_ARG) unless t (tensor or array; None passes) has exactly `shape`."""
-    if t is not None and _dims(t) != tuple(int(x) for x in shape):
+    if t is not None and _dims(t) != tuple(map(int, shape)):
         raise MG5Error(E_ARG, "%s has shape %s, expected %s" % (name, _dims(t), tuple(shape)))
 
 
@@ -328,9 +351,8 @@ def _box(t, name: str) -> tuple:
 
 
 def _stream(stream) -> int:
-    import torch
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
