@@ -98,15 +98,14 @@ struct Col {
     float cb1, Dyb1, Dzb1;         // plane p - 1 of B
 };
 
-// residual of the column's cell on plane p, given plane p + 1 (e2, b2)
-__device__ __forceinline__ float cell_resid(const Col &c, const PC &e2, const PC &b2, float fpc,
-                                            const CoefT<float> &cf)
+// op(B + e) - op(B) at the column's cell on plane p, given plane p + 1 (e2, b2)
+__device__ __forceinline__ float cell_op_col(const Col &c, const PC &e2, const PC &b2, const CoefT<float> &cf)
 {
     const Parts2 q = parts2_from_sums(
         __fadd_rn(e2.c, c.ce1), __fadd_rn(b2.c, c.cb1), c.e0.Y, c.b0.Y, c.e0.Z, c.b0.Z,
         __fsub_rn(e2.Dy, c.Dye1), __fsub_rn(b2.Dy, c.Dyb1), __fsub_rn(e2.Dz, c.Dze1),
         __fsub_rn(b2.Dz, c.Dzb1), c.e0.dyz, c.b0.dyz);
-    return __fsub_rn(fpc, cell_op_corr_parts(q, c.b0.c, c.e0.c, cf));
+    return cell_op_corr_parts(q, c.b0.c, c.e0.c, cf);
 }
 
 __device__ __forceinline__ void shift(Col &c, const PC &e2, const PC &b2)
@@ -121,11 +120,15 @@ __device__ __forceinline__ void shift(Col &c, const PC &e2, const PC &b2)
     c.b0 = b2;
 }
 
+// RHS: the FAS right-hand side of a coarse grid instead, f = (op(B + e) - op(B) + f) - m in place (a
+// CTA reads f in its own cells only), m at cptr; no statistics, and sides that the tiles do not divide
+// (what lies past the side is computed on the periodic images and not written).
+template <bool RHS>
 __global__ void __launch_bounds__(RT_THREADS, 2)
-    k_resid_restrict_march(const float *__restrict__ e, const float *__restrict__ f,
-                           const float *__restrict__ Bg, const double *__restrict__ cptr, int n,
-                           int ichunk, CoefT<float> cf, float *__restrict__ vc, float *__restrict__ v0c,
-                           float *__restrict__ rc, Moments *__restrict__ partials, Fin fin)
+    k_resid_restrict_march(const float *__restrict__ e, const float *f, const float *__restrict__ Bg,
+                           const double *__restrict__ cptr, int n, int ichunk, CoefT<float> cf,
+                           float *__restrict__ vc, float *__restrict__ v0c, float *rc,
+                           Moments *__restrict__ partials, Fin fin)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     ResidSmem &S = *reinterpret_cast<ResidSmem *>(smem_raw);
@@ -134,7 +137,7 @@ __global__ void __launch_bounds__(RT_THREADS, 2)
     const float cval = (float)(MG5_AT(cptr, 0));
     const int tid = threadIdx.x;
     const int jj = tid >> 4, pp = tid & 15;        // warp w: rows 2w (lanes 0-15), 2w+1
-    const int tk = n / RT_K, tiles = tk * (n / RT_J);
+    const int tk = (n + RT_K - 1) / RT_K, tiles = tk * ((n + RT_J - 1) / RT_J);
     const int items = tiles * ((n + ichunk - 1) / ichunk);
     MomAcc<float> acc;
 
@@ -175,8 +178,8 @@ __global__ void __launch_bounds__(RT_THREADS, 2)
                 const int r = w / (RT_K / 4), cc = w - r * (RT_K / 4);
                 src = f;
                 sp = S.F[0] + r * RT_K + cc * 4;
-                gj = j0 + r;
-                gk = k0 + cc * 4;
+                gj = wrap_once(j0 + r, n);
+                gk = wrap_once(k0 + cc * 4, n);
             }
             sdst[m] = (unsigned)__cvta_generic_to_shared(sp);
             gp[m] = src + (long long)wrap_once(q0, n) * n2 + (long long)gj * n + gk;
@@ -239,12 +242,20 @@ __global__ void __launch_bounds__(RT_THREADS, 2)
             plane_pair(S.E[s1] + offE, ea, eb);
             plane_pair(S.B[s1] + offE, ba, bb);
             const float2 fv = MG5_AT(reinterpret_cast<const float2 *>(S.F[s0] + offF), 0);
-            const float ra = cell_resid(ca, ea, ba, __fadd_rn(fv.x, cval), cf);
-            const float rb = cell_resid(cb, eb, bb, __fadd_rn(fv.y, cval), cf);
-            acc.add(ra);
-            acc.add(rb);
+            const float oa = cell_op_col(ca, ea, ba, cf), ob = cell_op_col(cb, eb, bb, cf);
+            const float ra = __fsub_rn(__fadd_rn(fv.x, cval), oa);
+            const float rb = __fsub_rn(__fadd_rn(fv.y, cval), ob);
             const float ua = ca.e0.c, ub = cb.e0.c;
-            if constexpr (!odd) {
+            if constexpr (!RHS) {
+                acc.add(ra);
+                acc.add(rb);
+            }
+            if constexpr (RHS) {
+                const int j = j0 + jj, k = k0 + 2 * pp;
+                if (j < n && k < n)
+                    MG5_AT(reinterpret_cast<float2 *>(rc + p * n2 + (long long)j * n + k), 0) =
+                        make_float2(__fsub_rn(__fadd_rn(oa, fv.x), cval), __fsub_rn(__fadd_rn(ob, fv.y), cval));
+            } else if constexpr (!odd) {
                 v0 = ua;
                 v1 = ub;
                 r0 = ra;
@@ -310,11 +321,15 @@ __global__ void __launch_bounds__(RT_THREADS, 2)
         acopy::wait<0>();
         __syncthreads();
     }
-    const Moments mom = block_moments(acc);
-    if (threadIdx.x == 0)
-        MG5_AT(partials, blockIdx.x) = mom;
-    if (fin.ls)
-        finalize_if_last(reinterpret_cast<double2 *>(partials), fin);
+    if constexpr (!RHS) {
+        const Moments mom = block_moments(acc);
+        if (threadIdx.x == 0)
+            MG5_AT(partials, blockIdx.x) = mom;
+        if (fin.ls)
+            finalize_if_last(reinterpret_cast<double2 *>(partials), fin);
+    } else if (blockIdx.x == 0 && threadIdx.x == 0) {
+        fin.ls->c = 0.0;
+    }
 }
 
 // CTAs of k_resid_restrict_march resident on the GPU at once (set by the preparation)
@@ -326,16 +341,19 @@ int g_resid_march_slots = 0;
 // together pass the 48 KiB default) and count its resident CTAs; once, outside any capture
 cudaError_t prepare_resid_march_kernel()
 {
-    cudaError_t e = cudaFuncSetAttribute(k_resid_restrict_march,
+    cudaError_t e = cudaFuncSetAttribute(k_resid_restrict_march<false>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sizeof(ResidSmem));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_resid_restrict_march<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(ResidSmem));
     int dev = 0, sms = 0, per_sm = 0;
     if (e == cudaSuccess)
         e = cudaGetDevice(&dev);
     if (e == cudaSuccess)
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_resid_restrict_march,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_resid_restrict_march<false>,
                                                           RT_THREADS, sizeof(ResidSmem));
     if (e == cudaSuccess)
         g_resid_march_slots = sms * (per_sm > 0 ? per_sm : 1);
@@ -344,19 +362,17 @@ cudaError_t prepare_resid_march_kernel()
 
 bool resid_march_ok(int n) { return n >= RT_K && n % RT_K == 0; }
 
-cudaError_t launch_resid_restrict_march(const float *e, const float *f, const double *cptr, int n,
-                                        CoefT<float> cf, float *vc, float *v0c, float *rc,
-                                        double2 *partials, int *nblocks, cudaStream_t st,
-                                        const float *B, const Fin &fin)
+// one CTA per resident slot (at most kReduceBlocks: one Moments partial each)
+static int march_slots()
 {
-    if (!resid_march_ok(n) || !B)
-        return cudaErrorInvalidValue;
-    // one CTA per resident slot (at most kReduceBlocks: one Moments partial each)
     const int slots = g_resid_march_slots > 0 ? g_resid_march_slots : 152;
-    const int g_max = slots < kReduceBlocks ? slots : kReduceBlocks;
-    const int tiles = (n / RT_K) * (n / RT_J);
-    // chunk length (even, at least 8 planes): the fewest plane steps per CTA, a chunk's two
-    // extra planes (i0 - 1 and i1) counted, over whole rounds of g_max items
+    return slots < kReduceBlocks ? slots : kReduceBlocks;
+}
+
+// chunk length (even, at least 8 planes): the fewest plane steps per CTA, a chunk's two
+// extra planes (i0 - 1 and i1) counted, over whole rounds of g_max items
+static int march_chunk(int n, int tiles, int g_max)
+{
     int ichunk = n, best = -1;
     for (int c = 8; c <= n; c += 2) {
         const long long items = (long long)tiles * ((n + c - 1) / c);
@@ -367,11 +383,43 @@ cudaError_t launch_resid_restrict_march(const float *e, const float *f, const do
             ichunk = c;
         }
     }
+    return ichunk;
+}
+
+cudaError_t launch_resid_restrict_march(const float *e, const float *f, const double *cptr, int n,
+                                        CoefT<float> cf, float *vc, float *v0c, float *rc,
+                                        double2 *partials, int *nblocks, cudaStream_t st,
+                                        const float *B, const Fin &fin)
+{
+    if (!resid_march_ok(n) || !B)
+        return cudaErrorInvalidValue;
+    const int g_max = march_slots();
+    const int tiles = (n / RT_K) * (n / RT_J);
+    const int ichunk = march_chunk(n, tiles, g_max);
     const long long items = (long long)tiles * ((n + ichunk - 1) / ichunk);
     const int g = (int)(items < g_max ? items : g_max);
-    k_resid_restrict_march<<<g, RT_THREADS, sizeof(ResidSmem), st>>>(
+    k_resid_restrict_march<false><<<g, RT_THREADS, sizeof(ResidSmem), st>>>(
         e, f, B, cptr, n, ichunk, cf, vc, v0c, rc, reinterpret_cast<Moments *>(partials), fin);
     *nblocks = g;
+    count_launch(1);
+    return cudaGetLastError();
+}
+
+// The gather kernel reads 38 values a cell, the march each plane of a column once: 96^3 15 -> 8 us, 128^3 32
+// -> 13, 256^3 242 -> 72; up to 64^3 both take ~6 us.
+bool rhs_march_ok(int n) { return n > 64 && n % 4 == 0; }
+
+cudaError_t launch_coarse_rhs_march(const float *v, float *f, const double *m_fine, LevelScal *ls, int n,
+                                    CoefT<float> cf, cudaStream_t st, const float *B)
+{
+    if (!rhs_march_ok(n) || !B)
+        return cudaErrorInvalidValue;
+    const int tiles = ((n + RT_K - 1) / RT_K) * ((n + RT_J - 1) / RT_J);
+    const int g_max = march_slots(), ichunk = march_chunk(n, tiles, g_max);
+    const long long items = (long long)tiles * ((n + ichunk - 1) / ichunk);
+    const int g = (int)(items < g_max ? items : g_max);
+    k_resid_restrict_march<true><<<g, RT_THREADS, sizeof(ResidSmem), st>>>(
+        v, f, B, m_fine, n, ichunk, cf, nullptr, nullptr, f, nullptr, Fin{ls, FIN_RESID, 0.0});
     count_launch(1);
     return cudaGetLastError();
 }

@@ -201,6 +201,11 @@ cudaError_t launch_resid_restrict_march(const float *e, const float *f, const do
                                         CoefT<float> cf, float *vc, float *v0c, float *rc,
                                         double2 *partials, int *nblocks, cudaStream_t st,
                                         const float *B, const Fin &fin = Fin());
+// the FAS right-hand side of the FP32 correction form as the same column march: f = op(v) + f - m_fine,
+// the grid's constant ls->c = 0; n > 64, a multiple of 4
+bool rhs_march_ok(int n);
+cudaError_t launch_coarse_rhs_march(const float *v, float *f, const double *m_fine, LevelScal *ls, int n,
+                                    CoefT<float> cf, cudaStream_t st, const float *B);
 // coarse = 8-child mean of fine
 template <typename T>
 cudaError_t launch_restrict(const T *fine, int n, T *coarse, cudaStream_t st);

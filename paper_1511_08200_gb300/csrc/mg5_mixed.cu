@@ -180,8 +180,10 @@ struct RunMix {
         }
         {
             ProfScope ps(sh.prof, PK_COARSE_RHS32, st, (double)(h->n[l]) * (h->n[l]) * (h->n[l]));
-            e = launch_coarse_rhs<float>(h->e[l], h->f[l], m(l - 1), c(l), h->n[l],
-                                         make_coef<float>(hl[l], p->alpha), st, h->B[l]);
+            const CoefT<float> cf = make_coef<float>(hl[l], p->alpha);
+            e = rhs_march_ok(h->n[l])
+                    ? launch_coarse_rhs_march(h->e[l], h->f[l], m(l - 1), ls(l), h->n[l], cf, st, h->B[l])
+                    : launch_coarse_rhs<float>(h->e[l], h->f[l], m(l - 1), c(l), h->n[l], cf, st, h->B[l]);
         }
         if (e != cudaSuccess)
             return fail("coarse_rhs32", e);
