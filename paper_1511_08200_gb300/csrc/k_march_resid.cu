@@ -25,7 +25,7 @@
 // ordered chunk-major and dealt round-robin, so the CTAs running at any time hold
 // neighbouring tiles at the same planes and share their halo rows in L2; the chunk length
 // is chosen so that the items fill whole rounds of the grid.  Periodic in i, j, k; n a
-// multiple of 32.
+// multiple of 32, or of 4 in the modes below that keep no statistics of their own.
 #include <type_traits>
 
 #include "mg5_async.cuh"
@@ -120,15 +120,20 @@ __device__ __forceinline__ void shift(Col &c, const PC &e2, const PC &b2)
     c.b0 = b2;
 }
 
+// RESTRICT: as above.
+// CHILDREN: without the statistics; the eight residuals of a coarse cell go to r8 in the order of its
+// children, and k_child_stats forms from them what the gather kernel does.
 // RHS: the FAS right-hand side of a coarse grid instead, f = (op(B + e) - op(B) + f) - m in place (a
-// CTA reads f in its own cells only), m at cptr; no statistics, and sides that the tiles do not divide
-// (what lies past the side is computed on the periodic images and not written).
-template <bool RHS>
+// CTA reads f in its own cells only), m at cptr.
+// CHILDREN and RHS take sides that the tiles do not divide (what lies past the side is computed on the
+// periodic images and not written).
+enum { RESTRICT, CHILDREN, RHS };
+template <int MODE>
 __global__ void __launch_bounds__(RT_THREADS, 2)
     k_resid_restrict_march(const float *__restrict__ e, const float *f, const float *__restrict__ Bg,
                            const double *__restrict__ cptr, int n, int ichunk, CoefT<float> cf,
                            float *__restrict__ vc, float *__restrict__ v0c, float *rc,
-                           Moments *__restrict__ partials, Fin fin)
+                           Moments *__restrict__ partials, Fin fin, float4 *__restrict__ r8)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     ResidSmem &S = *reinterpret_cast<ResidSmem *>(smem_raw);
@@ -246,11 +251,11 @@ __global__ void __launch_bounds__(RT_THREADS, 2)
             const float ra = __fsub_rn(__fadd_rn(fv.x, cval), oa);
             const float rb = __fsub_rn(__fadd_rn(fv.y, cval), ob);
             const float ua = ca.e0.c, ub = cb.e0.c;
-            if constexpr (!RHS) {
+            if constexpr (MODE == RESTRICT) {
                 acc.add(ra);
                 acc.add(rb);
             }
-            if constexpr (RHS) {
+            if constexpr (MODE == RHS) {
                 const int j = j0 + jj, k = k0 + 2 * pp;
                 if (j < n && k < n)
                     MG5_AT(reinterpret_cast<float2 *>(rc + p * n2 + (long long)j * n + k), 0) =
@@ -270,7 +275,7 @@ __global__ void __launch_bounds__(RT_THREADS, 2)
                 const float s3 = __shfl_down_sync(0xffffffffu, r1, 16);
                 const float s6 = __shfl_down_sync(0xffffffffu, ra, 16);
                 const float s7 = __shfl_down_sync(0xffffffffu, rb, 16);
-                if ((jj & 1) == 0) {
+                if ((jj & 1) == 0 && (MODE == RESTRICT || (j0 + jj < n && k0 + 2 * pp < n))) {
                     float sv = 0.f, sr = 0.f;
                     sv = __fadd_rn(sv, v0);
                     sv = __fadd_rn(sv, v1);
@@ -293,6 +298,10 @@ __global__ void __launch_bounds__(RT_THREADS, 2)
                     MG5_AT(vc, t) = mv;
                     MG5_AT(v0c, t) = mv;
                     MG5_AT(rc, t) = __fmul_rn(sr, 0.125f);
+                    if constexpr (MODE == CHILDREN) {
+                        MG5_AT(r8, 2 * t) = make_float4(r0, r1, s2, s3);
+                        MG5_AT(r8, 2 * t + 1) = make_float4(ra, rb, s6, s7);
+                    }
                 }
             }
             shift(ca, ea, ba);
@@ -321,15 +330,39 @@ __global__ void __launch_bounds__(RT_THREADS, 2)
         acopy::wait<0>();
         __syncthreads();
     }
-    if constexpr (!RHS) {
+    if constexpr (MODE == RESTRICT) {
         const Moments mom = block_moments(acc);
         if (threadIdx.x == 0)
             MG5_AT(partials, blockIdx.x) = mom;
         if (fin.ls)
             finalize_if_last(reinterpret_cast<double2 *>(partials), fin);
-    } else if (blockIdx.x == 0 && threadIdx.x == 0) {
+    } else if (MODE == RHS && blockIdx.x == 0 && threadIdx.x == 0) {
         fin.ls->c = 0.0;
     }
+}
+
+// The residual's statistics from the children's residuals, in the gather kernel's order (a coarse cell
+// a thread, the same blocks): the mean decides the FP32 rounding of all that follows it.
+__global__ void k_child_stats(const float4 *__restrict__ r8, long long total, Moments *__restrict__ partials, Fin fin)
+{
+    MomAcc<float> acc;
+    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
+         t += (long long)gridDim.x * blockDim.x) {
+        const float4 a = MG5_AT(r8, 2 * t), b = MG5_AT(r8, 2 * t + 1);
+        acc.add(a.x);
+        acc.add(a.y);
+        acc.add(a.z);
+        acc.add(a.w);
+        acc.add(b.x);
+        acc.add(b.y);
+        acc.add(b.z);
+        acc.add(b.w);
+    }
+    const Moments m = block_moments(acc);
+    if (threadIdx.x == 0)
+        MG5_AT(partials, blockIdx.x) = m;
+    if (fin.ls)
+        finalize_if_last(reinterpret_cast<double2 *>(partials), fin);
 }
 
 // CTAs of k_resid_restrict_march resident on the GPU at once (set by the preparation)
@@ -341,11 +374,14 @@ int g_resid_march_slots = 0;
 // together pass the 48 KiB default) and count its resident CTAs; once, outside any capture
 cudaError_t prepare_resid_march_kernel()
 {
-    cudaError_t e = cudaFuncSetAttribute(k_resid_restrict_march<false>,
+    cudaError_t e = cudaFuncSetAttribute(k_resid_restrict_march<RESTRICT>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sizeof(ResidSmem));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_resid_restrict_march<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(k_resid_restrict_march<CHILDREN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(ResidSmem));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_resid_restrict_march<RHS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sizeof(ResidSmem));
     int dev = 0, sms = 0, per_sm = 0;
     if (e == cudaSuccess)
@@ -353,7 +389,7 @@ cudaError_t prepare_resid_march_kernel()
     if (e == cudaSuccess)
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_resid_restrict_march<false>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_resid_restrict_march<RESTRICT>,
                                                           RT_THREADS, sizeof(ResidSmem));
     if (e == cudaSuccess)
         g_resid_march_slots = sms * (per_sm > 0 ? per_sm : 1);
@@ -398,10 +434,38 @@ cudaError_t launch_resid_restrict_march(const float *e, const float *f, const do
     const int ichunk = march_chunk(n, tiles, g_max);
     const long long items = (long long)tiles * ((n + ichunk - 1) / ichunk);
     const int g = (int)(items < g_max ? items : g_max);
-    k_resid_restrict_march<false><<<g, RT_THREADS, sizeof(ResidSmem), st>>>(
-        e, f, B, cptr, n, ichunk, cf, vc, v0c, rc, reinterpret_cast<Moments *>(partials), fin);
+    k_resid_restrict_march<RESTRICT><<<g, RT_THREADS, sizeof(ResidSmem), st>>>(
+        e, f, B, cptr, n, ichunk, cf, vc, v0c, rc, reinterpret_cast<Moments *>(partials), fin, nullptr);
     *nblocks = g;
     count_launch(1);
+    return cudaGetLastError();
+}
+
+// Restriction by the gather kernel -> march + statistics: 240^3 160 us -> 67 + 23, 176^3 71 -> 31 + 18, 120^3
+// 31 -> 14 + 14; at 104^3 25 -> 13 + 11 the second launch eats what the march saves.
+bool resid_children_ok(int n) { return n >= 112 && n % 4 == 0 && !resid_march_ok(n); }
+
+cudaError_t launch_resid_restrict_children(const float *e, const float *f, const double *cptr, int n,
+                                           CoefT<float> cf, float *vc, float *v0c, float *rc, float *work,
+                                           double2 *partials, int *nblocks, cudaStream_t st,
+                                           const float *B, const Fin &fin)
+{
+    if (!resid_children_ok(n) || !B)
+        return cudaErrorInvalidValue;
+    const int tiles = ((n + RT_K - 1) / RT_K) * ((n + RT_J - 1) / RT_J);
+    const int g_max = march_slots(), ichunk = march_chunk(n, tiles, g_max);
+    const long long items = (long long)tiles * ((n + ichunk - 1) / ichunk);
+    const int g = (int)(items < g_max ? items : g_max);
+    float4 *r8 = reinterpret_cast<float4 *>(work);
+    k_resid_restrict_march<CHILDREN><<<g, RT_THREADS, sizeof(ResidSmem), st>>>(
+        e, f, B, cptr, n, ichunk, cf, vc, v0c, rc, nullptr, Fin(), r8);
+    const long long total = (long long)(n / 2) * (n / 2) * (n / 2);
+    int gs = blocks_for(total);   // the blocks of launch_resid_restrict
+    if (gs > kReduceBlocks)
+        gs = kReduceBlocks;
+    k_child_stats<<<gs, kBlock, 0, st>>>(r8, total, reinterpret_cast<Moments *>(partials), fin);
+    *nblocks = gs;
+    count_launch(2);
     return cudaGetLastError();
 }
 
@@ -418,8 +482,8 @@ cudaError_t launch_coarse_rhs_march(const float *v, float *f, const double *m_fi
     const int g_max = march_slots(), ichunk = march_chunk(n, tiles, g_max);
     const long long items = (long long)tiles * ((n + ichunk - 1) / ichunk);
     const int g = (int)(items < g_max ? items : g_max);
-    k_resid_restrict_march<true><<<g, RT_THREADS, sizeof(ResidSmem), st>>>(
-        v, f, B, m_fine, n, ichunk, cf, nullptr, nullptr, f, nullptr, Fin{ls, FIN_RESID, 0.0});
+    k_resid_restrict_march<RHS><<<g, RT_THREADS, sizeof(ResidSmem), st>>>(
+        v, f, B, m_fine, n, ichunk, cf, nullptr, nullptr, f, nullptr, Fin{ls, FIN_RESID, 0.0}, nullptr);
     count_launch(1);
     return cudaGetLastError();
 }

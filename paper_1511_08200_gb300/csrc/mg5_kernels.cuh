@@ -201,6 +201,13 @@ cudaError_t launch_resid_restrict_march(const float *e, const float *f, const do
                                         CoefT<float> cf, float *vc, float *v0c, float *rc,
                                         double2 *partials, int *nblocks, cudaStream_t st,
                                         const float *B, const Fin &fin = Fin());
+// the same on sides that the march's tiles do not divide, with the gather kernel's statistics; work:
+// n^3 floats
+bool resid_children_ok(int n);
+cudaError_t launch_resid_restrict_children(const float *e, const float *f, const double *cptr, int n,
+                                           CoefT<float> cf, float *vc, float *v0c, float *rc, float *work,
+                                           double2 *partials, int *nblocks, cudaStream_t st,
+                                           const float *B, const Fin &fin = Fin());
 // the FAS right-hand side of the FP32 correction form as the same column march: f = op(v) + f - m_fine,
 // the grid's constant ls->c = 0; n > 64, a multiple of 4
 bool rhs_march_ok(int n);

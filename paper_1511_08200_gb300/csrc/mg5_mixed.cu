@@ -155,6 +155,10 @@ struct RunMix {
                 ? launch_resid_restrict_march(h->e[l], h->f[l], c(l), h->n[l], cf, h->e[l + 1],
                                               h->e0[l + 1], h->f[l + 1], sh.partials, &nb, st,
                                               h->B[l], fin)
+            : resid_children_ok(h->n[l])   // etmp, the sweeps' partner, is free here
+                ? launch_resid_restrict_children(h->e[l], h->f[l], c(l), h->n[l], cf, h->e[l + 1],
+                                                 h->e0[l + 1], h->f[l + 1], h->etmp[l], sh.partials,
+                                                 &nb, st, h->B[l], fin)
                 : launch_resid_restrict<float>(h->e[l], h->f[l], c(l), h->n[l], cf, h->e[l + 1],
                                                h->e0[l + 1], h->f[l + 1], sh.partials, &nb, st,
                                                h->B[l], fin);

@@ -1,4 +1,5 @@
-"""The FAS right-hand side of the FP32 correction form as a column march (coarse sides above 64)."""
+"""The FAS right-hand side of the FP32 correction form as a column march (coarse sides above 64), and its
+residual and restriction on fine sides that the march's tiles do not divide (112 and above)."""
 import numpy as np
 import pytest
 
@@ -8,9 +9,9 @@ from tests.gpu_common import ctx_fixture, dev, host, nominal
 pytestmark = pytest.mark.gpu
 
 
-# coarse sides 72, 88, 104, 128: last tiles of 4 .. 24 columns and 4 .. 8 rows, and full ones
-@pytest.mark.parametrize("n", [144, 176, 208, 256])
-def test_mixed_solve_with_the_marched_rhs(n):
+# fine sides: last tiles of 8 .. 16 columns and 0 .. 8 rows; coarse sides 60 (not marched), 72, 88, 104, 128
+@pytest.mark.parametrize("n", [120, 144, 176, 208, 256])
+def test_mixed_solve_with_the_marches(n):
     """The mixed solve reaches its tolerance and the FP64 solve's field: the residual is 1e-8 of the
     source; if all of it lay in the lowest mode, which holds at least 1e-3 of the source's norm,
     phi would be off by 1e-5."""
