@@ -369,23 +369,20 @@ cudaError_t launch_sweep_march(const float *in, float *out, const float *f, cons
     const int tk = (n + MT_K - 1) / MT_K, tj = (n + MT_J - 1) / MT_J, tiles = tk * tj;
     int ichunk = chunk;
     if (ichunk <= 0) {
-        if (tiles * (n / 16) >= 2 * 152) {
-            // about six waves of two CTAs per SM over 152 SMs, chunks of at least 16 planes
-            int chunks = (6 * 2 * 152 + tiles - 1) / tiles;
-            if (chunks > n / 16)
-                chunks = n / 16;
-            if (chunks < 1)
-                chunks = 1;
-            ichunk = (n + chunks - 1) / chunks;
-        } else {
-            // fewer CTAs than the GPU holds: the sweep takes as long as one CTA, a chunk's planes
-            // and the two before it one after the other, so the shortest chunk that fits at once (64^3:
-            // 12.4 us with chunks of 16 planes, 6.3 with 4).  Not below 4 planes: of shorter chunks
-            // half the work is the two extra planes, and boxes that share the GPU pay for it (a batch
-            // of 24 boxes of 32^3 .. 128^3: 13.9 ms with 16 planes, 13.6 with 4, 14.3 with 2)
-            ichunk = 4;
-            while (tiles * ((n + ichunk - 1) / ichunk) > 2 * 152)
-                ++ichunk;
+        // Equal CTAs, 2 x 152 at once: the sweep takes the rounds of CTAs times the plane steps of one, its
+        // planes, the two before them and about two for its first planes to arrive.  The chunk that
+        // makes this least (of 16 planes at most in 64^3 12.2 -> 5.6 us, 192^3 53 -> 48, 240^3 104 -> 94, 256^3
+        // 116 -> 107, 352^3 298 -> 259; 512^3 stays at 128).  Not below 4 planes: of
+        // shorter chunks half the work is the extra planes, and boxes that share the GPU pay for it
+        // (a batch of 24 boxes of 32^3 .. 128^3: 13.9 ms with 16 planes, 13.6 with 4, 14.3 with 2).
+        long long best = -1;
+        for (int c = n; c >= 4; --c) {
+            const long long ctas = (long long)tiles * ((n + c - 1) / c);
+            const long long cost = (ctas + 2 * kSMs - 1) / (2 * kSMs) * (c + 4);
+            if (best < 0 || cost < best) {
+                best = cost;
+                ichunk = c;
+            }
         }
     }
     if (ichunk > n)
