@@ -42,7 +42,9 @@ TOL64, TOLMIX = 1e-10, 1e-8
 NU_COARSE_CAP = 4        # coarsest-grid sweeps a visit in the FP64 solves of the step
 FP64_PEAK_TFLOPS = 2 * 2 * 152 * 2.07e9 / 1e12   # 2 FP64 FMA/clk/SM x 152 SMs x 2.07 GHz x 2 flop
 FP64_PEAK_SOURCE = ("derived FP64: 2 FMA/clk/SM x 152 SMs x 2.07 GHz x 2 flop = 1.259 TFLOP/s "
-                    "(MEASURED_PEAKS.json has no FP64 figure; an 8-chain FMA probe measured 1.195)")
+                    "(MEASURED_PEAKS.json has no FP64 figure; an 8-chain FMA probe measured 1.195); "
+                    "fractions above 1: sweeps on sides >= 48 compute FP64 results from exact FP32 "
+                    "pieces, not on the FP64 pipe")
 # The smoother's flops a cell update in the hot-path scope table's own count (about 60
 # arithmetic operations, one square root and one divide), reported beside the operation-by-
 # operation count of WORK for the same kernel.

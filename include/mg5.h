@@ -356,12 +356,13 @@ int mg5_solve_batch(mg5_ctx *ctx, int nbox, const double *const *delta, const in
 #define MG5_SWEEP_TWO_PASS 0
 #define MG5_SWEEP_FUSED    1
 #define MG5_SWEEP_MARCH    2   /* MG5_MIXED's FP32 correction-form sweep as a column march
-                                  (grid sides that are multiples of 32; others use the fused
-                                  kernel); in MG5_FP64 it reads as MG5_SWEEP_FUSED */
+                                  (grid sides that are multiples of 32; on others, and in
+                                  MG5_FP64, it reads as MG5_SWEEP_FUSED with chunk 0) */
 typedef struct {
     int form;    /* MG5_SWEEP_TWO_PASS, MG5_SWEEP_FUSED or MG5_SWEEP_MARCH */
     int block;   /* threads per block of the two-pass kernels (32 .. 1024, a multiple of 32) */
-    int chunk;   /* planes per CTA of the fused or march kernel (0 = automatic) */
+    int chunk;   /* planes per CTA of the fused or march kernel (0 = automatic: MG5_MIXED's fused form is
+                  * then the march on every side of 36 or more that is a multiple of 4) */
     float ms;    /* the tuner's median time of one sweep (0 when set by hand) */
 } mg5_schedule;
 /* Time every candidate schedule (two-pass with 32/64/128/256/512 threads, fused with

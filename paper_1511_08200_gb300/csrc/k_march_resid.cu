@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(RT_THREADS, 2)
         if (fin.ls)
             finalize_if_last(reinterpret_cast<double2 *>(partials), fin);
     } else if (MODE == RHS && blockIdx.x == 0 && threadIdx.x == 0) {
-        fin.ls->c = 0.0;
+        MG5_AT(fin.ls, 0).c = 0.0;
     }
 }
 

@@ -3,8 +3,8 @@
 // right-hand side (periodic grids and the finest grid of a refinement patch).
 //
 // What bounds them: the plain FP64 kernels sit at 84% of the FP64 pipe (2 lanes a clock per SM).
-// In the split arithmetic a cell costs FP32 and integer instructions instead (~330 a cell updated,
-// ~370 a residual, half of them packed), and the bound becomes instruction issue (57% busy) with
+// In the split arithmetic a cell costs FP32 and integer instructions instead (~495 a cell updated at 256^3,
+// ~370 a residual, half of them packed), and the bound becomes instruction issue (70% and 57% busy) with
 // the shared-memory (50%) and FMA (50%) pipes near behind.  Measured on GB300, plain FP64 -> split:
 // half-sweep 11.3 -> 5.5 us at 64^3, 64.4 -> 22.0 at 128^3, 500 -> 148 at 256^3; residual 26.6 ->
 // 12.3, 132 -> 41.5 and 994 -> 257 us.

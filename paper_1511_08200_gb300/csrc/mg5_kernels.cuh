@@ -185,8 +185,6 @@ cudaError_t launch_resid_restrict(const T *v, const T *f, const double *cptr, in
                                   CoefT<T> cf, T *vc, T *v0c, T *rc, double2 *partials,
                                   int *nblocks, cudaStream_t st, const T *B = nullptr,
                                   const Fin &fin = Fin());
-// the same for the FP32 correction form (B required) as a column march (k_march_resid.cu):
-// n a multiple of 32; the coarse values equal the gather kernel's to the bit
 // The bottom of an FP32 V-cycle in one CTA (k_bottom.cu): the visit of the periodic grids of sides
 // n[0 .. nlev - 1] (16, 8, 4 or 12, 6 or 8, 4: the last is the coarsest) in the correction form with
 // bases B; ls: the level scalars of n[0] and the grids below it.
@@ -195,6 +193,8 @@ cudaError_t prepare_bottom_kernel();
 cudaError_t launch_bottom(float *v, const float *f, const float *const *B, const int *n, int nlev,
                           const CoefT<float> *cf, const LevelScal *ls_up, LevelScal *ls, int nu1, int nu2,
                           int nu_coarse, double rtol, unsigned long long *clamp, int *sweeps, cudaStream_t st);
+// launch_resid_restrict for the FP32 correction form (B required) as a column march (k_march_resid.cu):
+// n a multiple of 32; the coarse values equal the gather kernel's to the bit
 bool resid_march_ok(int n);
 cudaError_t prepare_resid_march_kernel();
 cudaError_t launch_resid_restrict_march(const float *e, const float *f, const double *cptr, int n,
