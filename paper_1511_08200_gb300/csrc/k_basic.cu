@@ -292,8 +292,11 @@ cudaError_t launch_resid_restrict(const T *v, const T *f, const double *cptr, in
             return launch_split_resid_restrict(v, f, cptr, n, cf, vc, v0c, rc, partials, nblocks, st, fin);
         if (!B && 8 * work <= kChildMaxFine) {   // coarse grids of the FP64 solves
             const long long fine = 8 * work;
-            const int bf = block_spread(fine);
-            int gf = grid_spread(fine);
+            // One block an SM: with two or three (block_spread) the last block reads two or more partials a
+            // thread one after the other, and an SM may get three (32^3 14.1 -> 11.7 us, 24^3 16.4 -> 10.6)
+            const long long per = (fine + kSMs - 1) / kSMs;
+            const int bf = per >= kBlock ? kBlock : (int)((per + 31) & ~31ll);
+            int gf = (int)((fine + bf - 1) / bf);
             if (gf > cap)
                 gf = cap;
             k_resid_restrict_child<<<gf, bf, 0, st>>>(v, f, cptr, n, cf, vc, v0c, rc,
