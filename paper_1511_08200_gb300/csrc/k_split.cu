@@ -296,6 +296,14 @@ enum Out { RESTRICT, PLAIN, RHS };
 
 constexpr int RSUB = 4;
 
+// The statistics are FP32 sums of squares.  A residual of kStatMax u or more (a tile whose values are
+// 2^-25 of h^2 f and less) stays out of them: the cell (PLAIN) or the tile (RESTRICT) is computed
+// and counted in FP64.  With tiles of one sum at most 2^kStatGap apart, a difference from the shift
+// stays below 2^54 of its tile's unit and a tile's four squares below 2^110 of either unit, so the 2^14
+// tiles a thread has at 2048^3 stay finite.
+constexpr float kStatMax = 35184372088832.0f;   // 2^45
+constexpr int kStatGap = 8;
+
 struct ResidSmem {
     static constexpr int N = (RSUB + 2) * NJ * NK;
     float2 h[N], m[N], l[N];
@@ -400,16 +408,6 @@ __global__ void __launch_bounds__(THREADS, 3)
             T.template load<BOX>(v, v, i0, j0, k0, n0, n1, n2);
             const int emax = T.max_exponent();
             fast = tile_exponent(emax, cs, S.ex, eb, kap);
-            if (OUT == PLAIN && fast) {
-                // r may be written over f: an f beyond the pairs' range is looked for first
-                bool big = false;
-                const double lim = pow2(90 - kUnitBias + eb) * inv_h2;
-                const int j = j0 + warp, k = k0 + lane;
-                for (int m = 0; m < 2 * RSUB; ++m)
-                    if (i0 + m < n0 && j < n1 && k < n2)
-                        big = big || !(fabs(MG5_AT(f, ((long long)(i0 + m) * n1 + j) * n2 + k)) < lim);
-                fast = !__syncthreads_or(big || !(fabs(add) < lim));
-            }
             // a tile of zeros has r = f + add, which FP64 gives without rounding (the stopping
             // test of a source whose mean is far above its spread needs every bit of it)
             if (OUT != RHS)
@@ -435,7 +433,7 @@ __global__ void __launch_bounds__(THREADS, 3)
             return cell_residual(s, fm, cf);
         };
         if (fast) {
-            if (OUT != RHS && cnt > 0 && abs(eb - eb0) > 30)
+            if (OUT != RHS && cnt > 0 && abs(eb - eb0) > kStatGap)
                 flush();
             float Kt = cnt > 0 ? K * __int_as_float((eb0 - eb + 127) << 23) : 0.0f;
             Pair tsum{{0.0f, 0.0f}, {0.0f, 0.0f}}, tsq{{0.0f, 0.0f}, {0.0f, 0.0f}};
@@ -445,6 +443,7 @@ __global__ void __launch_bounds__(THREADS, 3)
             Pair ra{};
             P3 va{};
             bool bad = false;
+            int counted = min(max(n0 - i0, 0), RSUB) + min(max(n0 - i0 - RSUB, 0), RSUB);
             const bool in_a = col && i0 < n0;   // sides are even: a tile's planes come in pairs
             double fa = in_a ? MG5_AT(f, cell0) : 0.0,
                    fb = col && i0 + RSUB < n0 ? MG5_AT(f, cell0 + RSUB * plane_n) : 0.0;
@@ -464,18 +463,19 @@ __global__ void __launch_bounds__(THREADS, 3)
                                             (at(q + SI + 1) - at(q + SI - 1)) - (at(q - SI + 1) - at(q - SI - 1)),
                                             (at(q + NK + 1) - at(q + NK - 1)) - (at(q - NK + 1) - at(q - NK - 1))),
                                      pair_two(rha * to_u, rhb * to_u), kap);
-                // not finite, or an f beyond the pairs' range: the tile is done again in FP64
-                // (RHS, which overwrites f, recomputes the cell)
-                const bool bad_a = lva && !(fabsf(r.h.x) < 1e30f), bad_b = lvb && !(fabsf(r.h.y) < 1e30f);
+                // not finite, an f beyond the pairs' range, or too large for the statistics: the tile is
+                // done again in FP64 (RHS and PLAIN, which may write over f, recompute the cell)
+                constexpr float lim = OUT == RHS ? 1e30f : kStatMax;
+                const bool bad_a = lva && !(fabsf(r.h.x) < lim), bad_b = lvb && !(fabsf(r.h.y) < lim);
                 bad = bad || bad_a || bad_b;
                 if (OUT != RHS) {
                     if (!BOX && m == 0 && cnt == 0)
-                        Kt = fabsf(r.h.x) < 1e30f ? r.h.x : 0.0f;
+                        Kt = fabsf(r.h.x) < lim ? r.h.x : 0.0f;
                     Pair d = two_diff(r.h, both(Kt));
                     d.l = add2(d.l, r.l);
-                    if (!lva)
+                    if (!lva || bad_a)
                         d.h.x = d.l.x = 0.0f;
-                    if (!lvb)
+                    if (!lvb || bad_b)
                         d.h.y = d.l.y = 0.0f;
                     const Pair s = two_sum(tsum.h, d.h);
                     tsum.h = s.h;
@@ -504,23 +504,25 @@ __global__ void __launch_bounds__(THREADS, 3)
                         }
                     }
                 } else {
-                    if (rc) {
-                        if (lva) {
-                            double x = (unit_f64(r.h.x, eb) + unit_f64(r.l.x, eb)) * inv_h2;
-                            if (OUT == RHS && bad_a)
-                                x = slow(i0 + m, rha);
-                            MG5_AT(rc, cell) = OUT == RHS ? -x : x;
+                    const auto put = [&](float h, float l, bool redo, int i, double rh, long long q) {
+                        double x = (unit_f64(h, eb) + unit_f64(l, eb)) * inv_h2;
+                        if (redo) {
+                            x = slow(i, rh);
+                            if (OUT == PLAIN) {
+                                merge(Moments{1.0, x, 0.0, 0.0});
+                                --counted;
+                            }
                         }
-                        if (lvb) {
-                            double x = (unit_f64(r.h.y, eb) + unit_f64(r.l.y, eb)) * inv_h2;
-                            if (OUT == RHS && bad_b)
-                                x = slow(i0 + RSUB + m, rhb);
-                            MG5_AT(rc, cell + RSUB * plane_n) = OUT == RHS ? -x : x;
-                        }
-                    }
+                        if (rc)
+                            MG5_AT(rc, q) = OUT == RHS ? -x : x;
+                    };
+                    if (lva && (rc || bad_a))
+                        put(r.h.x, r.l.x, bad_a, i0 + m, rha, cell);
+                    if (lvb && (rc || bad_b))
+                        put(r.h.y, r.l.y, bad_b, i0 + RSUB + m, rhb, cell + RSUB * plane_n);
                 }
             }
-            if (OUT != RHS)
+            if (OUT == RESTRICT)
                 fast = !__syncthreads_or(bad);
             if (OUT != RHS && col && fast) {
                 if (cnt == 0) {
@@ -534,7 +536,7 @@ __global__ void __launch_bounds__(THREADS, 3)
                 t = two_sum(sq.h, mul2(tsq.h, both(up * up)));
                 sq.h = t.h;
                 sq.l = add2(sq.l, add2(t.l, mul2(tsq.l, both(up * up))));
-                cnt += min(max(n0 - i0, 0), RSUB) + min(max(n0 - i0 - RSUB, 0), RSUB);
+                cnt += counted;
             }
         }
         if (!fast) {
