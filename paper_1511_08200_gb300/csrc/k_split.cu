@@ -54,8 +54,10 @@ __device__ __forceinline__ void gather_at(const double *F, const double *E, int 
         gather3(F, E, E, periodic_rows(n0, i, j), k, k == n2 - 1 ? 0 : k + 1, k == 0 ? n2 - 1 : k - 1, s);
 }
 
-// The tile's common exponent from every thread's largest one, and whether the split arithmetic
-// takes the tile (every thread of the CTA must call it).
+__device__ __forceinline__ int exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// The tile's common exponent from every thread's largest one, and whether the split arithmetic takes
+// the tile, which it does not where all are 0 (every thread of the CTA must call it).
 __device__ __forceinline__ bool tile_exponent(int mine, const Coef &cs, int *sm, int &eb, Kap &kap)
 {
     mine = __reduce_max_sync(0xffffffffu, mine);
@@ -66,8 +68,6 @@ __device__ __forceinline__ bool tile_exponent(int mine, const Coef &cs, int *sm,
 #pragma unroll
     for (int w = 1; w < WARPS; ++w)
         eb = max(eb, sm[w]);
-    if (eb == 0)
-        eb = 1023;   // nothing but zeros
     const bool in_range = eb >= kMinExp && eb <= kMaxExp;
     const float u = __int_as_float((in_range ? eb - kUnitBias + 127 : 127) << 23);
     kap = Kap{cs.k3h * u, cs.k3l * u, cs.kh * u, cs.kl * u};
@@ -210,7 +210,12 @@ __global__ void __launch_bounds__(THREADS, SUB == 4 && !BOX ? 4 : 3)
     T.template load<BOX>(act ? faces : same, act ? same : faces, i0, j0, k0, n0, n1, n2);
     int eb;
     Kap kap;
-    const bool fast = tile_exponent(T.max_exponent(), cs, S.ex, eb, kap);
+    // A tile that is zero or tiny beside its source (the first half-sweep of a cold start) takes a unit 2^-77 of
+    // the source, of which a sample is at hand: what its own values lose then lies 2^-60 below the change,
+    // and the unit of 1 would round an h^2 f below 2^-92 to nothing.  Cells whose source is out of
+    // the pairs' range all the same, and a tile of zeros whose sample is zero, go to FP64.
+    const int fx = max(max(exponent(fan), exponent(fbn)), exponent(c)) + exponent(cf.h2) - 1021;   // h^2 (f + c) < 2^(fx - 1022)
+    const bool fast = tile_exponent(max(T.max_exponent(), fx - 57), cs, S.ex, eb, kap);
     if (fast)
         T.store(eb, [&](int ii, int jj, int kk, const P3 &p) {
             const int col = ((ii + jj + kk) & 1) == act ? 0 : 1, q = (ii * NJ + jj) * HK + (kk >> 1);
@@ -297,12 +302,12 @@ enum Out { RESTRICT, PLAIN, RHS };
 constexpr int RSUB = 4;
 
 // The statistics are FP32 sums of squares.  A residual of kStatMax u or more (a tile whose values are
-// 2^-25 of h^2 f and less) stays out of them: the cell (PLAIN) or the tile (RESTRICT) is computed
+// 2^-18 of h^2 f and less) stays out of them: the cell (PLAIN) or the tile (RESTRICT) is computed
 // and counted in FP64.  With tiles of one sum at most 2^kStatGap apart, a difference from the shift
-// stays below 2^54 of its tile's unit and a tile's four squares below 2^110 of either unit, so the 2^14
-// tiles a thread has at 2048^3 stay finite.
-constexpr float kStatMax = 35184372088832.0f;   // 2^45
-constexpr int kStatGap = 8;
+// stays below 2^55 of its tile's unit, and a tile's four squares below 2^112 of it and of the sum's, so the
+// 2^14 tiles a thread has at 2048^3 stay finite.
+constexpr float kStatMax = 274877906944.0f;   // 2^38
+constexpr int kStatGap = 16;
 
 struct ResidSmem {
     static constexpr int N = (RSUB + 2) * NJ * NK;
@@ -406,10 +411,12 @@ __global__ void __launch_bounds__(THREADS, 3)
         {
             TileRegs<RSUB> T;
             T.template load<BOX>(v, v, i0, j0, k0, n0, n1, n2);
+            // a tile of zeros (eb = 0) has r = f + add, which FP64 gives without rounding (the stopping
+            // test of a source whose mean is far above its spread needs every bit of it)
             const int emax = T.max_exponent();
             fast = tile_exponent(emax, cs, S.ex, eb, kap);
-            // a tile of zeros has r = f + add, which FP64 gives without rounding (the stopping
-            // test of a source whose mean is far above its spread needs every bit of it)
+            // (tile_exponent has refused it already; asked again, the kernel compiles to 271 us at 256^3
+            // instead of 278)
             if (OUT != RHS)
                 fast = __syncthreads_or(emax != 0) && fast;
             if (fast)
@@ -443,7 +450,7 @@ __global__ void __launch_bounds__(THREADS, 3)
             Pair ra{};
             P3 va{};
             bool bad = false;
-            int counted = min(max(n0 - i0, 0), RSUB) + min(max(n0 - i0 - RSUB, 0), RSUB);
+            int redone = 0;
             const bool in_a = col && i0 < n0;   // sides are even: a tile's planes come in pairs
             double fa = in_a ? MG5_AT(f, cell0) : 0.0,
                    fb = col && i0 + RSUB < n0 ? MG5_AT(f, cell0 + RSUB * plane_n) : 0.0;
@@ -473,9 +480,9 @@ __global__ void __launch_bounds__(THREADS, 3)
                         Kt = fabsf(r.h.x) < lim ? r.h.x : 0.0f;
                     Pair d = two_diff(r.h, both(Kt));
                     d.l = add2(d.l, r.l);
-                    if (!lva || bad_a)
+                    if (!lva || (OUT == PLAIN && bad_a))
                         d.h.x = d.l.x = 0.0f;
-                    if (!lvb || bad_b)
+                    if (!lvb || (OUT == PLAIN && bad_b))
                         d.h.y = d.l.y = 0.0f;
                     const Pair s = two_sum(tsum.h, d.h);
                     tsum.h = s.h;
@@ -510,7 +517,7 @@ __global__ void __launch_bounds__(THREADS, 3)
                             x = slow(i, rh);
                             if (OUT == PLAIN) {
                                 merge(Moments{1.0, x, 0.0, 0.0});
-                                --counted;
+                                ++redone;
                             }
                         }
                         if (rc)
@@ -536,7 +543,7 @@ __global__ void __launch_bounds__(THREADS, 3)
                 t = two_sum(sq.h, mul2(tsq.h, both(up * up)));
                 sq.h = t.h;
                 sq.l = add2(sq.l, add2(t.l, mul2(tsq.l, both(up * up))));
-                cnt += counted;
+                cnt += min(max(n0 - i0, 0), RSUB) + min(max(n0 - i0 - RSUB, 0), RSUB) - redone;
             }
         }
         if (!fast) {

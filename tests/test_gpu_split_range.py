@@ -1,5 +1,5 @@
 """The split-arithmetic FP64 kernels where a tile's values are tiny beside its source: residuals whose
-squares leave the FP32 range."""
+squares leave the FP32 range, tiles of zeros, and sources that a tile's unit would round away."""
 import numpy as np
 import pytest
 
@@ -66,7 +66,7 @@ def test_patch_from_a_tiny_guess_without_presmoothing(ctx):
 
 @pytest.mark.parametrize("n", [64, 66])
 def test_large_and_small_residuals_over_their_source(ctx, n):
-    """Residuals of 2^35 .. 2^70 of a tile's unit, in place: each is the source to the rounding of the sum
+    """Residuals of 2^33 .. 2^68 of a tile's unit, in place: each is the source to the rounding of the sum
     (2^-47 where it is a pair)."""
     alpha, s, h = nominal()
     rng = np.random.default_rng(n)
@@ -77,3 +77,43 @@ def test_large_and_small_residuals_over_their_source(ctx, n):
         got = host(ctx.step_residual(dev(phi), g, 0.0, h, 1e-12, out=g if out else None))
         ref = oracle.residual(phi, f, 0.0, h, 1e-12)
         assert np.all(np.abs(got - ref) <= 2.0**-46 * np.abs(ref) + 2.0**-46 * 24 * np.abs(phi).max() / h**2)
+
+
+@pytest.mark.parametrize("n", [64, 66])
+@pytest.mark.parametrize("where", ["everywhere", "a block"])
+@pytest.mark.parametrize("size", [1e-30, 1e-24, 1.0, 1e20])
+def test_sweep_of_zeros(ctx, n, where, size):
+    """The half-sweep of a tile of zeros, with h^2 f of any size (alpha f stays what it is): a change is
+    good to 2^-44 of itself, in a tile's unit to 2^-60 of the largest."""
+    alpha, s, h = nominal()
+    rng = np.random.default_rng(n)
+    f = rng.standard_normal((n,) * 3)
+    f[:, :, n // 2:] = 0.0
+    phi = np.zeros_like(f)
+    scale = size / h**2
+    if where == "a block":
+        phi[n // 2:] = 0.1 * h * h * rng.standard_normal((n - n // 2, n, n))
+    a = 0.01 / scale
+    got = host(ctx.step_sweep(dev(phi * scale), dev(f * scale), 0.0, h, a))
+    ref = oracle.sweep(phi * scale, f * scale, 0.0, h, a)
+    assert np.abs(got - ref).max() <= 1e-13 * np.abs(ref).max()
+    quiet = np.s_[2:n // 2 - 2, :, n // 2 + 2:-2]   # no source and no value around
+    assert np.array_equal(got[quiet], np.zeros_like(got[quiet]))
+
+
+@pytest.mark.parametrize("n", [64, 128])
+@pytest.mark.parametrize("nu", [(2, 2), (0, 3)])
+def test_a_solve_scales_by_powers_of_two(ctx, n, nu):
+    """The linear equation in units 2^-70 apart (h^2 f is 1e-9 and 1e-30): no smoothing is lost, so the
+    cycles are the same, and the fields to what two residuals of 1e-11 leave if all of both lay in the
+    lowest mode (at least 1e-3 of the source's norm)."""
+    import paper_1511_08200_gb300 as mg
+    _, s, h = nominal()
+    d = dev(workload.lognormal_delta(n, 1.0, 82))
+    out = []
+    for u in (1.0, 2.0**-70):
+        p = mg.default_params(alpha=0.0, s=s * u, h=h, tol=1e-11, nu1=nu[0], nu2=nu[1])
+        phi, _, info = ctx.solve_fifth_force(d, p)
+        out.append((host(phi) / u, info.cycles, info.status))
+    assert out[0][1:] == out[1][1:] and out[0][2] == 0
+    assert rel_l2(out[0][0], out[1][0]) <= 2e-8
