@@ -501,6 +501,14 @@ int mg5_step_sweep(mg5_ctx *ctx, const double *phi_in, double *phi_out, const do
 int mg5_step_resid_restrict_f32(mg5_ctx *ctx, const float *e, const float *f, const float *B,
                                 double c, int N, double h, double alpha, int variant, float *ec,
                                 float *rc, double *stats, void *stream);
+/* One coarse visit of the mixed mode's FP32 V-cycle, grid N and all below it: e = R e and f = R r of the
+ * grid above, m its mean r, B the base on grid N; p gives h (of grid N), alpha, nu1, nu2, nu_coarse and
+ * omega.  e_out: the corrected e, c_out (host): the grid's compatibility constant.  e, f, B, e_out:
+ * device, N^3 floats.  variant 0: one launch a step by the kernels that gather; 1: as the solves run it.
+ * Both give the same values, to the bit where no grid of 8^3 lies below N or is it (its mean residual
+ * is summed in another order).  Allocates and frees a hierarchy of N; synchronises the stream. */
+int mg5_step_visit_f32(mg5_ctx *ctx, const float *e, const float *f, const float *B, double m, int N,
+                       const mg5_params *p, int variant, float *e_out, double *c_out, void *stream);
 /* The same sweep by the fused kernel (one read and one write of phi per cell). */
 int mg5_step_sweep_fused(mg5_ctx *ctx, const double *phi_in, double *phi_out, const double *f,
                          double c, int N, double h, double alpha, void *stream);

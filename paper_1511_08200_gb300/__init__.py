@@ -161,6 +161,7 @@ _sigs = {
     "mg5_step_operator": ([_P, _P, _c_int, _c_double, _c_double, _P, _P], _c_int),
     "mg5_step_resid_restrict_f32": ([_P, _P, _P, _P, _c_double, _c_int, _c_double, _c_double, _c_int,
                                      _P, _P, _P, _P], _c_int),
+    "mg5_step_visit_f32": ([_P, _P, _P, _P, _c_double, _c_int, _P, _c_int, _P, _P, _P], _c_int),
     "mg5_step_residual": ([_P, _P, _P, _c_double, _c_int, _c_double, _c_double, _P, _P], _c_int),
     "mg5_step_restrict": ([_P, _P, _c_int, _P, _P], _c_int),
     "mg5_step_prolong_add": ([_P, _P, _c_int, _P, _P], _c_int),
@@ -676,6 +677,20 @@ class Context:
             n, h, alpha, 1 if march else 0, _ptr(ec, "float32", dv), _ptr(rc, "float32", dv), st,
             _stream(stream)))
         return ec, rc, (st[0], st[1])
+
+    def step_visit_f32(self, e, f, base, m: float, params: Params, plain=False, stream=None):
+        """mg5_step_visit_f32: (corrected e, c) of a coarse visit of the FP32 V-cycle; plain: by the
+        kernels that gather, a launch a step."""
+        import torch
+        n = _cube(e, "e")
+        self._cubes(n, f=f, base=base)
+        out = torch.empty_like(e)
+        c = _c_double()
+        dv = self.device
+        self._check(_lib.mg5_step_visit_f32(
+            self._h, _ptr(e, "float32", dv), _ptr(f, "float32", dv), _ptr(base, "float32", dv), m, n,
+            ctypes.byref(params), 0 if plain else 1, _ptr(out, "float32", dv), ctypes.byref(c), _stream(stream)))
+        return out, c.value
 
     def step_operator(self, phi, h: float, alpha: float, out=None, stream=None):
         import torch

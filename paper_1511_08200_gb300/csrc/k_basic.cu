@@ -477,6 +477,16 @@ __global__ void k_prolong_add(const T *__restrict__ vc, const T *__restrict__ v0
 }
 
 template <typename T>
+cudaError_t launch_prolong_gather(const T *vc, const T *v0c, int nc, T *vf, double *c_fine,
+                                  const double *c_coarse, cudaStream_t st)
+{
+    const long long work = (long long)nc * nc * nc;
+    k_prolong_add<T><<<grid_spread(work), block_spread(work), 0, st>>>(vc, v0c, nc, vf, c_fine, c_coarse);
+    count_launch(1);
+    return cudaGetLastError();
+}
+
+template <typename T>
 cudaError_t launch_prolong_add(const T *vc, const T *v0c, int nc, T *vf, double *c_fine,
                                const double *c_coarse, cudaStream_t st)
 {
@@ -485,10 +495,7 @@ cudaError_t launch_prolong_add(const T *vc, const T *v0c, int nc, T *vf, double 
     // tile's two phases cost more (56^3 fine, FP64: 6.9 us, 8.5 as tiles; 64^3: 9.0 and 8.7)
     if (nc > 32)
         return launch_prolong_tile<T>(vc, v0c, nc, vf, c_fine, c_coarse, st);
-    const long long work = (long long)nc * nc * nc;
-    k_prolong_add<T><<<grid_spread(work), block_spread(work), 0, st>>>(vc, v0c, nc, vf, c_fine, c_coarse);
-    count_launch(1);
-    return cudaGetLastError();
+    return launch_prolong_gather<T>(vc, v0c, nc, vf, c_fine, c_coarse, st);
 }
 
 // --------------------------------------------------------------------------
@@ -1180,6 +1187,8 @@ cudaError_t launch_patch_residual(const double *phi, const double *fint, double 
     template cudaError_t launch_restrict<T>(const T *, int, T *, cudaStream_t);                    \
     template cudaError_t launch_coarse_rhs<T>(const T *, T *, const double *, double *, int,       \
                                               CoefT<T>, cudaStream_t, const T *);                  \
+    template cudaError_t launch_prolong_gather<T>(const T *, const T *, int, T *, double *,           \
+                                               const double *, cudaStream_t);                      \
     template cudaError_t launch_prolong_add<T>(const T *, const T *, int, T *, double *,           \
                                                const double *, cudaStream_t);                      \
     template cudaError_t launch_coarsest<T>(T *, T *, const T *, int, CoefT<T>, double *, int,     \

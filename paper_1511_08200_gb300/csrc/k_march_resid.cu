@@ -123,10 +123,11 @@ __device__ __forceinline__ void shift(Col &c, const PC &e2, const PC &b2)
 // RESTRICT: as above.
 // CHILDREN: without the statistics; the eight residuals of a coarse cell go to r8 in the order of its
 // children, and k_child_stats forms from them what the gather kernel does.
-// RHS: the FAS right-hand side of a coarse grid instead, f = (op(B + e) - op(B) + f) - m in place (a
-// CTA reads f in its own cells only), m at cptr.
+// RHS: the FAS right-hand side of a coarse grid instead, f = (op(B + e) - op(B) + f) - m in place, m at
+// cptr.  A CTA copies f of its own cells only: not the planes on either side of its chunk, nor the periodic
+// images past the side, which other CTAs overwrite meanwhile.
 // CHILDREN and RHS take sides that the tiles do not divide (what lies past the side is computed on the
-// periodic images and not written).
+// periodic images, RHS with any f, and not written).
 enum { RESTRICT, CHILDREN, RHS };
 template <int MODE>
 __global__ void __launch_bounds__(RT_THREADS, 2)
@@ -149,7 +150,7 @@ __global__ void __launch_bounds__(RT_THREADS, 2)
     // this thread's 16-byte chunks of a plane (e, B: rows j0-1.., f: the tile)
     unsigned sdst[RT_CPT];
     const float *gp[RT_CPT];
-    bool has[RT_CPT];
+    bool has[RT_CPT], own[RT_CPT];   // own: RHS, a chunk of f inside the grid
 #pragma unroll
     for (int m = 0; m < RT_CPT; ++m) {
         const int c = tid + m * RT_THREADS;
@@ -185,16 +186,22 @@ __global__ void __launch_bounds__(RT_THREADS, 2)
                 sp = S.F[0] + r * RT_K + cc * 4;
                 gj = wrap_once(j0 + r, n);
                 gk = wrap_once(k0 + cc * 4, n);
+                own[m] = j0 + r < n && k0 + cc * 4 < n;   // (n is a multiple of 4)
             }
             sdst[m] = (unsigned)__cvta_generic_to_shared(sp);
             gp[m] = src + (long long)wrap_once(q0, n) * n2 + (long long)gj * n + gk;
         }
         int qn = wrap_once(q0, n);
+        int left = -1;   // RHS: planes of the chunk that have been copied (the first plane lies below it)
         auto issue_next = [&](int s) {
+            const bool inside = MODE != RHS || (left >= 0 && left < i1 - i0);
+            ++left;
 #pragma unroll
             for (int m = 0; m < RT_CPT; ++m)
                 if (has[m]) {
                     const int c = tid + m * RT_THREADS;
+                    if (MODE == RHS && c >= 2 * RT_CH_EB && !(inside && own[m]))
+                        continue;
                     const unsigned stride = c < 2 * RT_CH_EB ? RPL * 4 : FPL * 4;
                     acopy::copy16(sdst[m] + (unsigned)s * stride, gp[m]);
                 }

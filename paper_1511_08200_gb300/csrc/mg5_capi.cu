@@ -2757,6 +2757,21 @@ int mg5_step_resid_restrict_f32(mg5_ctx *ctx, const float *e, const float *f, co
     return MG5_OK;
 }
 
+int mg5_step_visit_f32(mg5_ctx *ctx, const float *e, const float *f, const float *B, double m, int N,
+                       const mg5_params *p, int variant, float *e_out, double *c_out, void *stream)
+{
+    if (!ctx || !e || !f || !B || !e_out || !c_out || variant < 0 || variant > 1 || check_size(N) != MG5_OK ||
+        check_params(p) != MG5_OK)
+        return MG5_E_ARG;
+    CK(cudaSetDevice(ctx->device));
+    MixedHier *h = nullptr;
+    RET(alloc_mixed(N, ctx->budget, &ctx->held, &h, &ctx->err));
+    const MixedShared sh{ctx->partials, ctx->ls, ctx->cnt, ctx->h_rel, &ctx->prof, nullptr};
+    const int rc = step_visit_mixed(h, sh, e, f, B, m, p, variant == 0, e_out, c_out, (cudaStream_t)stream, &ctx->err);
+    free_mixed(h, &ctx->held);
+    return rc;
+}
+
 int mg5_step_sweep_fused(mg5_ctx *ctx, const double *in, double *out, const double *f, double c,
                          int N, double h, double alpha, void *stream)
 {

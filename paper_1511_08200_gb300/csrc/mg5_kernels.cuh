@@ -225,6 +225,10 @@ cudaError_t launch_coarse_rhs(const T *vc, T *fc, const double *m_fine, double *
 template <typename T>
 cudaError_t launch_prolong_tile(const T *vc, const T *v0c, int nc, T *vf, double *c_fine,
                                 const double *c_coarse, cudaStream_t st);
+// ... a thread a coarse cell, which gathers: any nc
+template <typename T>
+cudaError_t launch_prolong_gather(const T *vc, const T *v0c, int nc, T *vf, double *c_fine,
+                                  const double *c_coarse, cudaStream_t st);
 template <typename T>
 cudaError_t launch_prolong_add(const T *vc, const T *v0c, int nc, T *vf, double *c_fine,
                                const double *c_coarse, cudaStream_t st);

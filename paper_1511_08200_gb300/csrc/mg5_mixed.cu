@@ -99,6 +99,7 @@ struct RunMix {
     std::string *err;
     double hl[kMixMaxLevels];
     long long cu = 0;  // cell updates of the non-coarsest sweeps
+    bool plain = false;   // the gather kernels everywhere, one launch a step (step_visit_mixed)
 
     LevelScal *ls(int l) { return sh.ls + kInnerBase + l; }
     double *c(int l) { return &ls(l)->c; }
@@ -116,8 +117,12 @@ struct RunMix {
         const CoefT<float> cf = make_coef<float>(hl[l], p->alpha, omega_of(p));
         int dev = 0;
         cudaGetDevice(&dev);
-        cudaError_t e = launch_sweep_sched<float>(sweep_schedule(dev, MG5_MIXED, h->n[l]), h->e[l],
-                                                  h->etmp[l], h->f[l], c(l), h->n[l], cf,
+        SweepSchedule sched = sweep_schedule(dev, MG5_MIXED, h->n[l]);
+        if (plain && sched.form) {
+            sched.form = 1;
+            sched.chunk = 16;   // the fused kernel, not the march
+        }
+        cudaError_t e = launch_sweep_sched<float>(sched, h->e[l], h->etmp[l], h->f[l], c(l), h->n[l], cf,
                                                   &sh.cnt->clamped, st, h->B[l]);
         if (e != cudaSuccess)
             return fail("sweep32", e);
@@ -151,11 +156,11 @@ struct RunMix {
         const CoefT<float> cf = make_coef<float>(hl[l], p->alpha);
         const Fin fin{ls(l), FIN_RESID, n3};
         cudaError_t e =
-            resid_march_ok(h->n[l])
+            !plain && resid_march_ok(h->n[l])
                 ? launch_resid_restrict_march(h->e[l], h->f[l], c(l), h->n[l], cf, h->e[l + 1],
                                               h->e0[l + 1], h->f[l + 1], sh.partials, &nb, st,
                                               h->B[l], fin)
-            : resid_children_ok(h->n[l])   // etmp, the sweeps' partner, is free here
+            : !plain && resid_children_ok(h->n[l])   // etmp, the sweeps' partner, is free here
                 ? launch_resid_restrict_children(h->e[l], h->f[l], c(l), h->n[l], cf, h->e[l + 1],
                                                  h->e0[l + 1], h->f[l + 1], h->etmp[l], sh.partials,
                                                  &nb, st, h->B[l], fin)
@@ -168,7 +173,7 @@ struct RunMix {
     int coarse_visit(int l)
     {
         cudaError_t e;
-        if (bottom_ok(h->n + l, h->nlev - l)) {
+        if (!plain && bottom_ok(h->n + l, h->nlev - l)) {
             // this grid and those below it in a single launch (k_bottom.cu)
             ProfScope ps(sh.prof, PK_COARSEST32, st);
             CoefT<float> cf[kMixMaxLevels];
@@ -185,7 +190,7 @@ struct RunMix {
         {
             ProfScope ps(sh.prof, PK_COARSE_RHS32, st, (double)(h->n[l]) * (h->n[l]) * (h->n[l]));
             const CoefT<float> cf = make_coef<float>(hl[l], p->alpha);
-            e = rhs_march_ok(h->n[l])
+            e = !plain && rhs_march_ok(h->n[l])
                     ? launch_coarse_rhs_march(h->e[l], h->f[l], m(l - 1), ls(l), h->n[l], cf, st, h->B[l])
                     : launch_coarse_rhs<float>(h->e[l], h->f[l], m(l - 1), c(l), h->n[l], cf, st, h->B[l]);
         }
@@ -202,8 +207,10 @@ struct RunMix {
             return rc;
         {
             ProfScope ps(sh.prof, PK_PROLONG32, st, (double)(h->n[l]) * (h->n[l]) * (h->n[l]));
-            e = launch_prolong_add<float>(h->e[l + 1], h->e0[l + 1], h->n[l + 1], h->e[l], c(l),
-                                          c(l + 1), st);
+            e = plain ? launch_prolong_gather<float>(h->e[l + 1], h->e0[l + 1], h->n[l + 1], h->e[l], c(l),
+                                                     c(l + 1), st)
+                      : launch_prolong_add<float>(h->e[l + 1], h->e0[l + 1], h->n[l + 1], h->e[l], c(l),
+                                                  c(l + 1), st);
         }
         if (e != cudaSuccess)
             return fail("prolong32", e);
@@ -411,6 +418,29 @@ int phase_finish(MixedHier *h, const MixedShared &sh, double *phi, cudaStream_t 
 }
 
 }  // namespace
+
+int step_visit_mixed(MixedHier *h, const MixedShared &sh, const float *e, const float *f, const float *B,
+                     double m, const mg5_params *p, bool plain, float *e_out, double *c_out, cudaStream_t st,
+                     std::string *err)
+{
+    RunMix R{h, sh, p, st, err, {}, 0, plain};
+    for (int l = 0; l < h->nlev; ++l)
+        R.hl[l] = p->h * (double)(1 << l);
+    const size_t b = (size_t)h->N * h->N * h->N * sizeof(float);
+    CKM(cudaMemcpyAsync(h->e[0], e, b, cudaMemcpyDeviceToDevice, st));
+    CKM(cudaMemcpyAsync(h->f[0], f, b, cudaMemcpyDeviceToDevice, st));
+    CKM(cudaMemcpyAsync(h->B[0], B, b, cudaMemcpyDeviceToDevice, st));
+    for (int l = 1; l < h->nlev; ++l)
+        CKM(launch_restrict<float>(h->B[l - 1], h->n[l - 1], h->B[l], st));
+    CKM(cudaMemsetAsync(sh.ls, 0, sizeof(LevelScal) * kScalSlots, st));
+    CKM(cudaMemcpyAsync(R.m(-1), &m, sizeof(double), cudaMemcpyHostToDevice, st));
+    if (int rc = R.coarse_visit(0))
+        return rc;
+    CKM(cudaMemcpyAsync(e_out, h->e[0], b, cudaMemcpyDeviceToDevice, st));
+    CKM(cudaMemcpyAsync(c_out, R.c(0), sizeof(double), cudaMemcpyDeviceToHost, st));
+    CKM(cudaStreamSynchronize(st));
+    return MG5_OK;
+}
 
 int solve_mixed(MixedHier *h, const MixedShared &sh, const double *delta, const mg5_params *p,
                 double *phi, mg5_info *info, cudaStream_t st, std::string *err, bool zero_start)

@@ -93,6 +93,12 @@ void free_mixed(MixedHier *m, size_t *held);
 // zero_start: phi holds zeros (not a warm start), so the first residual skips the stencil
 int solve_mixed(MixedHier *m, const MixedShared &sh, const double *delta, const mg5_params *p,
                 double *phi, mg5_info *info, cudaStream_t st, std::string *err, bool zero_start);
+// One coarse visit of an FP32 V-cycle (grid N and all below it): e, f hold the restricted correction
+// and residual, m the residual mean of the grid above, B the base; e_out the corrected e, c_out the
+// grid's constant.  plain: by the gather kernels, a launch a step.  Synchronises.
+int step_visit_mixed(MixedHier *m, const MixedShared &sh, const float *e, const float *f, const float *B,
+                     double mean, const mg5_params *p, bool plain, float *e_out, double *c_out, cudaStream_t st,
+                     std::string *err);
 // Record, into the graph being captured on `st`, a whole mixed solve (phi
 // zero start) with its defect-correction loop as a WHILE node whose body is
 // captured on `st_body`; then gauge and (if grad) the force.  The loop state
