@@ -343,16 +343,19 @@ int mg5_solve_batch(mg5_ctx *ctx, int nbox, const double *const *delta, const in
                     void *stream);
 
 /* ------------------------------------------------------------ autotuner
- * The smoother's schedule changes speed, not values: the two-pass sweep (a red
+ * The smoother's schedule changes speed, not the method: the two-pass sweep (a red
  * and a black kernel, `block` threads per block) or the fused plane-march
  * (one kernel, each CTA marching over `chunk` planes; 0 = enough CTAs for
- * several waves) apply the same cell update of Sec. 3.1 to the same snapshot.
+ * several waves) apply the same cell update of Sec. 3.1 to the same snapshot, and
+ * agree to rounding.  MG5_FP64 sides of 48 and more have one kernel: every schedule
+ * there gives the same values to the bit, at the same speed.
  * The table is process-wide, keyed by (device, precision, grid side n); solves,
  * batch captures and MG5_GRAPH captures read it when they start (a captured
  * graph keeps the schedule it was captured with).  Defaults: FP64 two-pass with
  * 256 threads a block, or on grids too small to give each of the 152 SMs two such
- * blocks the multiple of 32 (at least 32) that does; the mixed mode's FP32 correction form as a column march where n is
- * a multiple of 32, else fused where n >= 32 and n % 4 == 0. */
+ * blocks the multiple of 32 (at least 32) that does (of effect below 48); the mixed
+ * mode's FP32 correction form as a column march where n is a multiple of 32, else
+ * fused with chunk 0 where n > 32 and n % 4 == 0, which is the march there too. */
 #define MG5_SWEEP_TWO_PASS 0
 #define MG5_SWEEP_FUSED    1
 #define MG5_SWEEP_MARCH    2   /* MG5_MIXED's FP32 correction-form sweep as a column march
@@ -366,8 +369,9 @@ typedef struct {
     float ms;    /* the tuner's median time of one sweep (0 when set by hand) */
 } mg5_schedule;
 /* Time every candidate schedule (two-pass with 32/64/128/256/512 threads, fused with
- * 8/16/32 planes where it fits, and for MG5_MIXED the column march with automatic,
- * 16, 32, 64 or 128 planes where it fits) on a synthetic field of each grid side of the
+ * 8/16/32 planes where it fits, for MG5_MIXED also automatic, and the column march with
+ * automatic, 16, 32, 64 or 128 planes where it fits; for MG5_FP64 sides of 48 and more the
+ * one kernel there is) on a synthetic field of each grid side of the
  * hierarchy of N (coarsest excluded) on ctx's device and stream, and record the
  * fastest; sides already in the table are kept.  Synchronises `stream`; must not
  * run during a stream capture.  Allocates (and frees) 3-4 grids of the side. */

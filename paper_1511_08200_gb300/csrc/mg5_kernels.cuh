@@ -136,7 +136,16 @@ cudaError_t launch_sweep_march(const float *in, float *out, const float *f, cons
                                unsigned long long *clamp, cudaStream_t st, int chunk = 0);
 cudaError_t prepare_march_kernel();
 
-// How one grid side is swept (speed only: every schedule computes the same values).
+// The split arithmetic (k_split.cu) takes FP64 grids from these sizes up; smaller ones keep the plain
+// FP64 kernels.  Sweeps: a 48^3 half-sweep takes 4.0 us against 6.5, a 32^3 solve lost 4% (16 tiles).
+// Residuals: 64^3 takes 12.3 us against 26.6, and below 64^3 the FP64 residual is the more exact one
+// (the stopping test is made of it).
+constexpr int kSplitMinSweep = 48, kSplitMinResid = 64;
+constexpr long long kSplitMinPatch = 40 * 40 * 40;   // cells of a patch's finest grid
+
+// How one grid side is swept (speed only: every schedule applies the same cell update to the same
+// snapshot; the kernels differ in rounding, FP32's fused and march kernels not even in that).
+// FP64 sides of kSplitMinSweep and more have one kernel, whatever the schedule says.
 struct SweepSchedule {
     int form = 0;     // 0: two-pass, 1: fused (chunk 0, FP32: the march where it is as exact and faster),
                       // 2: column march (FP32 correction form)
@@ -162,7 +171,8 @@ cudaError_t launch_sweep_sched(const SweepSchedule &s, const T *in, T *out, cons
         if (s.form == 2 && B && march_ok(n))
             return launch_sweep_march(in, out, f, B, cptr, n, cf, clamp, st, s.chunk);
     }
-    if ((s.form == 1 || s.form == 2) && fused_ok<T>(n)) {
+    const bool one_kernel = sizeof(T) == 8 && !B && n >= kSplitMinSweep;
+    if ((s.form == 1 || s.form == 2) && fused_ok<T>(n) && !one_kernel) {
         // the same values as the fused kernel, faster; a set chunk of planes means that kernel
         if constexpr (sizeof(T) == 4) {
             if (B && !march_ok(n) && march_ragged_ok(n) && !(s.form == 1 && s.chunk))
@@ -249,11 +259,6 @@ cudaError_t launch_coarsest(T *v, T *tmp, const T *f, int n, CoefT<T> cf, double
                             const T *B = nullptr);
 
 // ---- FP64 kernels in split arithmetic (k_split.cu, mg5_split.cuh)
-// Smaller sides keep the plain FP64 kernels.  Sweeps: a 48^3 half-sweep takes 4.0 us against 6.5, a
-// 32^3 solve lost 4% (16 tiles).  Residuals: 64^3 takes 12.3 us against 26.6, and below 64^3 the
-// FP64 residual is the more exact one (the stopping test is made of it).
-constexpr int kSplitMinSweep = 48, kSplitMinResid = 64;
-constexpr long long kSplitMinPatch = 40 * 40 * 40;   // cells of a patch's finest grid
 cudaError_t prepare_split_kernels();
 // snapshot red-black sweep (two launches), as launch_sweep
 cudaError_t launch_split_sweep(const double *in, double *out, const double *f, const double *cptr, int n,

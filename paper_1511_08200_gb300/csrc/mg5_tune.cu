@@ -1,11 +1,11 @@
 // mg5_tune.cu -- autotuner of the sweep schedule (host runtime, C ABI in mg5.h).
 //
-// The smoother's schedule changes speed, not values: the two-pass sweep with
-// 32 .. 512 threads per block (by default 256, fewer on coarse grids so that their
+// The smoother's schedule changes speed (and rounding), not the method: the two-pass sweep
+// with 32 .. 512 threads per block (by default 256, fewer on coarse grids so that their
 // warps reach more SMs), the column march of the mixed mode's FP32 sweep
 // (k_march.cu), or the fused plane-march with 8 .. 32 planes per
 // CTA, all apply the same cell update to the same snapshot (the sweep of
-// Sec. 3.1).  Which is fastest depends on the grid side (waves over the 152
+// Sec. 3.1).  FP64 sides of 48 and more have one kernel (k_split.cu) and one candidate.  Which is fastest depends on the grid side (waves over the 152
 // SMs, shared-memory rings vs L2 reuse) and on the precision (the FP64 sweep
 // is bound by the FP64 pipe, the mixed mode's FP32 sweep by issue and
 // memory).  The tuner times every candidate on a synthetic field of the side
@@ -81,6 +81,10 @@ struct TuneBufs {
 std::vector<SweepSchedule> candidates(int precision, int n)
 {
     std::vector<SweepSchedule> v;
+    if (precision == MG5_FP64 && n >= kSplitMinSweep) {
+        v.push_back(default_schedule(precision, n));
+        return v;
+    }
     for (int b : {32, 64, 128, 256, 512}) {
         SweepSchedule s;
         s.form = 0;
