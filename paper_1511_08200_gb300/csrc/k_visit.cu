@@ -801,11 +801,9 @@ unsigned magic(int d) { return d < 2 ? 0u : (unsigned)((0x100000000ull + d - 1) 
 
 }  // namespace
 
-static bool g_visit_fits = false;   // a cluster of kVisitCtas CTAs can be resident (set by the preparation)
-
 bool visit_plan(const int (*q)[3], int nlev, bool box, VisitArgs *A)
 {
-    if (!g_visit_fits || nlev < 1 || nlev > kVisitLevels)
+    if (nlev < 1 || nlev > kVisitLevels)
         return false;
     int quads = 0;   // of 16 bytes
     for (int l = 0; l < nlev; ++l) {
@@ -871,10 +869,10 @@ void visit_level_consts(VisitLevel *L, const CoefT<double> &cf, double w)
     }
 }
 
-cudaError_t prepare_visit_kernels()
+cudaError_t prepare_visit_kernels(bool *fits)
 {
     cudaError_t e = cudaSuccess;
-    bool fits = true;
+    *fits = true;
     for (const void *k : {(const void *)k_visit<false>, (const void *)k_visit<true>}) {
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kVisitSmem);
@@ -885,10 +883,8 @@ cudaError_t prepare_visit_kernels()
         int n = 0;
         if (e == cudaSuccess)
             e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
-        fits = fits && n > 0;
+        *fits = *fits && n > 0;
     }
-    if (e == cudaSuccess)
-        g_visit_fits = fits;
     return e;
 }
 

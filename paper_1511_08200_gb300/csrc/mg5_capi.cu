@@ -185,6 +185,7 @@ struct mg5_ctx {
     unsigned long long graph_clock = 0;
     double2 *partials = nullptr;
     LevelScal *ls = nullptr;        // kScalSlots slots
+    bool visit_fits = false;        // the device holds k_visit.cu's cluster
     SolveCounters *cnt = nullptr;
     double *h_rel = nullptr;        // pinned host scalars
     // staging for MG5_HOST_IO and patch scratch
@@ -654,7 +655,7 @@ struct Run64 {
     bool visit(int l, cudaError_t *e)
     {
         const int n = h->n[l];
-        if ((long long)n * n * n > kVisitCells || h->n[h->nlev - 1] >= kSpectralMinSide)
+        if (!ctx->visit_fits || (long long)n * n * n > kVisitCells || h->n[h->nlev - 1] >= kSpectralMinSide)
             return false;
         VisitArgs A = {};
         int q[kMaxLevels][3];
@@ -971,7 +972,7 @@ int mg5_create(mg5_ctx **out, int device, size_t budget)
     if (e == cudaSuccess)
         e = prepare_fused_kernels();
     if (e == cudaSuccess)
-        e = prepare_visit_kernels();
+        e = prepare_visit_kernels(&ctx->visit_fits);
     if (e == cudaSuccess)
         e = prepare_bottom_kernel();
     if (e != cudaSuccess) {
@@ -1426,7 +1427,7 @@ struct RunPatch {
     bool visit(int l, cudaError_t *e)
     {
         VisitArgs A = {};
-        if (mk[0] || (long long)int_cells(h->q[l]) > kVisitCells || !visit_plan(h->q + l, h->nlev - l, true, &A))
+        if (!ctx->visit_fits || mk[0] || (long long)int_cells(h->q[l]) > kVisitCells || !visit_plan(h->q + l, h->nlev - l, true, &A))
             return false;
         ProfScope ps(&ctx->prof, PK_COARSEST64, st);
         for (int k = l; k < h->nlev; ++k) {

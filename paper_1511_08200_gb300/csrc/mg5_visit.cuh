@@ -42,11 +42,13 @@ struct VisitArgs {
     VisitLevel lev[kVisitLevels];
 };
 
-// Fills sides, distribution and shared-memory layout; false: the grids do not fit.
+// Fills sides, distribution and shared-memory layout; false: the grids do not fit.  (Whether the device
+// takes the cluster at all is the context's to know: prepare_visit_kernels.)
 bool visit_plan(const int (*q)[3], int nlev, bool box, VisitArgs *A);
 // ... and a level's constants (w: extrapolation weight of a box's ghosts).
 void visit_level_consts(VisitLevel *L, const CoefT<double> &cf, double w);
-cudaError_t prepare_visit_kernels();
+// Sets the kernels' attributes on the current device; *fits: it can hold a cluster of kVisitCtas CTAs.
+cudaError_t prepare_visit_kernels(bool *fits);
 cudaError_t launch_visit(const VisitArgs &A, bool box, cudaStream_t st);
 
 }  // namespace mg5
