@@ -163,6 +163,11 @@ int mg5_release(mg5_ctx *ctx);
  * (default) spins, which answers sooner but holds a CPU core.  Many threads
  * solving at once on few cores (the server's workers) should sleep. */
 int mg5_set_blocking_wait(mg5_ctx *ctx, int on);
+/* Debugging aid: how many bits above the largest value it starts from the first attempt at an FP64
+ * coarse visit leaves its values (default 2; -64 .. 2).  A value that outgrows them makes the visit
+ * start over with eight bits more, six times at most, after which it leaves no correction.  Solves
+ * captured before keep what they were captured with. */
+int mg5_set_visit_headroom(mg5_ctx *ctx, int bits);
 /* on = 1: a solve (or batch, or MG5_GRAPH capture) first tunes the sweep schedule
  * of every grid side of its hierarchy that has no entry yet (mg5_autotune), before
  * any capture begins.  Default 0: untuned sides use the default schedule. */

@@ -138,6 +138,7 @@ _sigs = {
     "mg5_server_destroy": ([_P], _c_int),
     "mg5_server_get_stats": ([_P, _P], _c_int),
     "mg5_set_blocking_wait": ([_P, _c_int], _c_int),
+    "mg5_set_visit_headroom": ([_P, _c_int], _c_int),
     "mg5_set_autotune": ([_P, _c_int], _c_int),
     "mg5_autotune": ([_P, _c_int, _c_int, _P], _c_int),
     "mg5_schedule_get": ([_c_int, _c_int, _c_int, _P], _c_int),
@@ -407,6 +408,10 @@ class Context:
     def set_blocking_wait(self, on: bool = True):
         """mg5_set_blocking_wait: sleep (True) or spin (False, default) while waiting for the GPU."""
         self._check(_lib.mg5_set_blocking_wait(self._h, 1 if on else 0))
+
+    def set_visit_headroom(self, bits: int = 2):
+        """mg5_set_visit_headroom: bits the first attempt at an FP64 coarse visit leaves its values."""
+        self._check(_lib.mg5_set_visit_headroom(self._h, bits))
 
     def _check(self, rc: int, allow=(OK,)):
         if rc not in allow:

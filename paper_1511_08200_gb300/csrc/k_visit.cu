@@ -19,7 +19,8 @@
 //  * the residual, its restriction and the correction pass between grids as pairs through the grids'
 //    own global buffers (L2);
 //  * a value that outgrows its unit raises a flag: at the end all CTAs agree and repeat the visit
-//    with eight bits more.
+//    with eight bits more, six times at most.  Where that is not enough, or values are not finite, the
+//    visit leaves no correction: v = v0, c = 0 (the grid above keeps its own sweeps and its residual test).
 //
 // Measured on GB300 (a visit, launches -> cluster): top grid 16^3 periodic 130 -> 67 us, with the
 // 32^3 patch's 16^3 grid below it 100 -> 46 us.  A half-sweep takes 2.1 kclk at 4^3, 2.95 at 8^3 and 3.6
@@ -98,6 +99,7 @@ struct Visit {
     unsigned clamps = 0;
     int sweeps = 0;
     int eb = 0;      // the visit's exponent: u = 2^(eb - kUnitBias)
+    bool finite = true;   // of the top grid's values
     int turn = 0;    // of the reduction buffers
 
     // the planes [i0, i0 + np) of level l this CTA owns
@@ -223,6 +225,13 @@ struct Visit {
     {
         return split1((unsigned)__double2hiint(x), (unsigned)__double2loint(x), eb);
     }
+    // ... of a value that may not fit the unit
+    __device__ __forceinline__ P1 split_checked(double x)
+    {
+        if (((__double2hiint(x) >> 20) & 0x7ff) > eb)
+            S.flag = 1;
+        return split_f64(x);
+    }
     // the change of a cell since the visit began
     __device__ __forceinline__ Pr change(const P1 &now, double v0) const { return pair_of(now - split_f64(v0)); }
     // kappa of a grid: a quarter of the parent's, whose h is half of its own
@@ -281,7 +290,8 @@ struct Visit {
     __device__ __forceinline__ Pr weight(const VisitLevel &L, int m) const { return Pr{L.w[m - 1][0], L.w[m - 1][1]}; }
     // The ghosts after a half-sweep (k_patch_half's order): after the red one every ghost of the
     // sweep's result, after the black one those of the black cells.  a0, a1: the arrays of the two
-    // colours' values; d0, d1: of the ghosts.  (v0 does not change any more: it may come from L1.)
+    // colours' values; d0, d1: of the ghosts.  (v0 does not change any more, and the barrier after it was
+    // written is an acquire: it may come from L1.)
     __device__ __forceinline__ void ghosts_follow(const VisitLevel &L, const Own &o, bool black, int a0, int a1,
                                                   int d0, int d1)
     {
@@ -318,7 +328,7 @@ struct Visit {
         };
         const auto see = [&](double v, double r) {
             const int ef = (__double2hiint(r) >> 20) & 0x7ff, ev = (__double2hiint(v) >> 20) & 0x7ff;
-            emax = max(emax, max(ev, ef > 0 ? min(ef + grow, 2046) : 0));
+            emax = max(emax, max(ev, ef == 2047 ? 2047 : (ef > 0 ? min(ef + grow, 2046) : 0)));
         };
 #pragma unroll
         for (int m = 0; m < kHold; ++m) {
@@ -353,6 +363,7 @@ struct Visit {
         for (int r = 0; r < kVisitCtas; ++r)
             emax = max(emax, S.ebs[r]);
         eb = min(max((emax == 0 ? 1023 : emax) + margin, 200), 1800);
+        finite = emax < 2047;
         if (tid == 0) {
             // (one thread: an FP64 instruction of every warp would take 256 clocks)
             const double k1 = L.k * pow2d(eb - kUnitBias), k3 = 3.0 * k1;
@@ -363,7 +374,7 @@ struct Visit {
         }
         const auto keep = [&](int t, double v, double r) {
             const int q = div_by(t, L.m2), k = t - q * L.n2, p = div_by(q, L.m1), j = q - p * L.n1;
-            put(L, o, arr((o.i0 + p + j + k) & 1, 0), p, j, k, split_f64(v));
+            put(L, o, arr((o.i0 + p + j + k) & 1, 0), p, j, k, split_checked(v));
             const Pr F = in_units(L, r);
             Fat(L, p, j, k) = make_float2(F.h, F.l);
         };
@@ -398,7 +409,7 @@ struct Visit {
             const auto add2 = [&](int a) { return add_pair(Pr{q[a].x, q[a].y}, Pr{q[a + 1].x, q[a + 1].y}); };
             const Pr r = add_pair(add_pair(add2(0), add2(2)), add_pair(add2(4), add2(6)));
             Fat(L, p, j, k) = make_float2(0.5f * r.h, 0.5f * r.l);
-            put(L, o, arr((i + j + k) & 1, 0), p, j, k, split_f64(x));
+            put(L, o, arr((i + j + k) & 1, 0), p, j, k, split_checked(x));
         });
     }
     // ... then the ghosts' fixed values and c = 0
@@ -409,7 +420,7 @@ struct Visit {
 #pragma unroll 1
         for (int t = tid; t < ng; t += VT) {
             const Ghost g = ghost(L, o, t);
-            array(L, arr(g.ca ^ (g.m & 1), 0))[at(L, g.p, g.j, g.k)] = st(split_f64(v0_at(L, o.i0 + g.p, g.j, g.k)));
+            array(L, arr(g.ca ^ (g.m & 1), 0))[at(L, g.p, g.j, g.k)] = st(split_checked(v0_at(L, o.i0 + g.p, g.j, g.k)));
         }
         if (tid == 0)
             S.c[L.id] = Pr{0.0f, 0.0f};
@@ -426,7 +437,7 @@ struct Visit {
         const Pr c = S.c[L.id];
         Pr mean{0.0f, 0.0f};
         if (!BOX && mode == RHS)   // (the parent's unit u / h^2 is four of L's)
-            mean = L.id > 0 ? scale(Pm, 4.0f) : in_units(L, *A.m_up);
+            mean = L.id > 0 ? scale(Pm, 4.0f) : in_units(L, MG5_AT(A.m_up, 0));
         sum = Pr{0.0f, 0.0f};
         sq = Pr{0.0f, 0.0f};
         cells(L, o, [&](int p, int j, int k) {
@@ -489,7 +500,7 @@ struct Visit {
                 const Pr r = resid(lin, add_pair(F, c), kap);
                 const Pr d = neg(mul_pair(root_change(lin, r, kap, clamps), Pr{L.wh, L.wl}));
                 const P1 x = add_change(now, d);
-                if (fabsf(x.h) > kPieceMax || fabsf(d.h) > 2.0f * kPieceMax)
+                if (!(fabsf(x.h) <= kPieceMax && fabsf(d.h) <= 2.0f * kPieceMax))   // (NaN too)
                     S.flag = 1;
                 put(L, o, ad, p, j, k, x);
             }
@@ -598,7 +609,7 @@ struct Visit {
             const Pr y0 = three(line(a[0], a[1]), line(a[0], n[1])), y1 = three(line(n[0], a[1]), line(n[0], n[1]));
             const Pr d = scale(three(y0, y1), 1.0f / 64.0f);
             const P1 x = add_change(centre(L, b, p, j, k, col), d);
-            if (fabsf(x.h) > kPieceMax || fabsf(d.h) > 2.0f * kPieceMax)
+            if (!(fabsf(x.h) <= kPieceMax && fabsf(d.h) <= 2.0f * kPieceMax))
                 S.flag = 1;
             put(L, o, arr(col, b), p, j, k, x);   // (a box's ghosts follow in the next sweep, as in k_patch_half)
         });
@@ -633,7 +644,7 @@ struct Visit {
     // once: inlined at each of their uses it outgrew the instruction cache (a half-sweep of 8^3 took
     // 4400 clocks).
     enum Step { ENTER, DOWNWARD, COARSEST, UPWARD, DONE };
-    __device__ __forceinline__ bool run(int margin)
+    __device__ __forceinline__ bool run(int margin, bool last_attempt)
     {
         if (tid == 0)
             S.flag = 0;
@@ -723,7 +734,7 @@ struct Visit {
         int any = 0;
         for (int r = 0; r < kVisitCtas; ++r)
             any |= S.flags[r];
-        if (any && margin < 2 + 8 * kRestarts)
+        if (any && !last_attempt && finite)
             return false;
         // the top grid's iterate and c
         const VisitLevel &L = A.lev[0];
@@ -743,7 +754,7 @@ struct Visit {
                 const int i = o.i0 + p;
                 if (t < n)
                     MG5_AT(L.v, vcell(L, i, j, k)) =
-                        v0[m] + to_f64(change(centre(L, b, p, j, k, (i + j + k) & 1), v0[m]), eb);
+                        any ? v0[m] : v0[m] + to_f64(change(centre(L, b, p, j, k, (i + j + k) & 1), v0[m]), eb);
             }
         }
         const int ng = ghost_count(L, o);
@@ -753,11 +764,11 @@ struct Visit {
             if (i >= 0 && i < L.n0 && (g.p < 0 || g.p >= o.np))
                 continue;
             const Pr e = change(centre(L, b, g.pa, g.ja, g.ka, g.ca), v0_at(L, o.i0 + g.pa, g.ja, g.ka));
-            MG5_AT(L.v, vcell(L, i, g.j, g.k)) =
-                v0_at(L, i, g.j, g.k) + to_f64(mul_pair(weight(L, g.m), e), eb);
+            const double vg = v0_at(L, i, g.j, g.k);
+            MG5_AT(L.v, vcell(L, i, g.j, g.k)) = any ? vg : vg + to_f64(mul_pair(weight(L, g.m), e), eb);
         }
         if (!BOX && rank == 0 && tid == 0)
-            *A.c_out = to_f64(S.c[0], eb) / L.h2;
+            MG5_AT(A.c_out, 0) = any ? 0.0 : to_f64(S.c[0], eb) / L.h2;
         return true;
     }
 };
@@ -769,10 +780,10 @@ __global__ void __launch_bounds__(VT, 1) k_visit(const __grid_constant__ VisitAr
     __shared__ VisitShared S;
     cg::cluster_group cluster = cg::this_cluster();
     Visit<BOX> V{A, S, visit_sm, cluster, (int)cluster.block_rank(), (int)threadIdx.x};
-    for (int margin = 2;; margin += 8) {
+    for (int it = 0;; ++it) {
         V.clamps = 0;
         V.sweeps = 0;
-        if (V.run(margin))
+        if (V.run(A.headroom + 8 * it, it == kRestarts))
             break;
     }
     if (V.clamps)

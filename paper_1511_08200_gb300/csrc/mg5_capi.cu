@@ -186,6 +186,7 @@ struct mg5_ctx {
     double2 *partials = nullptr;
     LevelScal *ls = nullptr;        // kScalSlots slots
     bool visit_fits = false;        // the device holds k_visit.cu's cluster
+    int visit_headroom = kVisitHeadroom;
     SolveCounters *cnt = nullptr;
     double *h_rel = nullptr;        // pinned host scalars
     // staging for MG5_HOST_IO and patch scratch
@@ -678,6 +679,7 @@ struct Run64 {
         A.nu2 = p->nu2;
         A.nu_coarse = p->nu_coarse;
         A.rtol = kCoarseRtol;
+        A.headroom = ctx->visit_headroom;
         A.m_up = m(l - 1);
         A.c_out = c(l);
         A.clamp = &cntb->clamped;
@@ -1067,6 +1069,14 @@ int mg5_set_blocking_wait(mg5_ctx *ctx, int on)
     return MG5_OK;
 }
 
+int mg5_set_visit_headroom(mg5_ctx *ctx, int bits)
+{
+    if (!ctx || bits < -64 || bits > kVisitHeadroom)
+        return MG5_E_ARG;
+    ctx->visit_headroom = bits;
+    return MG5_OK;
+}
+
 int mg5_cached_bytes(mg5_ctx *ctx, int N, int precision, size_t *extra)
 {
     if (!ctx || !extra)
@@ -1444,6 +1454,7 @@ struct RunPatch {
         A.nu2 = p->nu2;
         A.nu_coarse = p->nu_coarse;
         A.rtol = kCoarseRtol;
+        A.headroom = ctx->visit_headroom;
         A.clamp = &cntb->clamped;
         A.sweeps = &cntb->coarse_sweeps;
         *e = launch_visit(A, true, st);

@@ -12,6 +12,7 @@ constexpr int kVisitLevels = 6;
 constexpr int kVisitCells = 20000;
 constexpr int kVisitCoarsest = 2048;          // cells of a coarsest grid CTA 0 iterates
 constexpr int kVisitSmem = 222 * 1024;        // dynamic shared memory a CTA may use
+constexpr int kVisitHeadroom = 2;             // bits: rounding, and a nonlinear correction above the linear one
 
 struct VisitLevel {
     int id, n0, n1, n2;    // interior sides
@@ -34,6 +35,7 @@ struct VisitLevel {
 
 struct VisitArgs {
     int nlev, nu1, nu2, nu_coarse, smem;
+    int headroom;          // bits above the largest value that the first attempt's unit leaves
     double rtol;
     const double *m_up;    // mean residual of the grid above (periodic)
     double *c_out;         // c of the top grid (periodic)
