@@ -830,8 +830,9 @@ struct RefineSrc {
 // FP64 bound as a sum of eight weighted values (~40 FP64 operations a cell: 21 us for 66^3): the
 // weights are 3/4 and 1/4 of the nearer and the farther centre on each axis, so the axes go one
 // after the other as 3 near + far with the three factors 1/4 in one exact 1/64 at the end, eight
-// FP64 operations a cell.  Indices in 32 bits where the arrays have fewer than 2^31 cells
-// (a 64-bit division is ~100 instructions).
+// FP64 operations a cell.  (A result that is not finite may be an overflow of the 64-fold value: it is
+// formed again with the factors 1/4 at each axis.)  Indices in 32 bits where the arrays have fewer than
+// 2^31 cells (a 64-bit division is ~100 instructions).
 template <typename Int>
 __global__ void k_refine(const double *__restrict__ phic, RefineSrc src, int o0, int o1, int o2,
                          int d0, int d1, int d2, int g, double *__restrict__ fine)
@@ -878,7 +879,18 @@ __global__ void k_refine(const double *__restrict__ phic, RefineSrc src, int o0,
         }
         y[a] = fma(3.0, x[0], x[1]);
     }
-    MG5_AT(fine, t) = fma(3.0, y[0], y[1]) * (1.0 / 64.0);
+    double v = fma(3.0, y[0], y[1]) * (1.0 / 64.0);
+    if ((__double2hiint(v) & 0x7ff00000) == 0x7ff00000) {
+        const auto mean = [](double near, double far) { return fma(0.75, near, 0.25 * far); };
+#pragma unroll 1
+        for (int a = 0; a < 2; ++a) {
+            const Int r0 = ((Int)at[0][a] * src.c1 + at[1][0]) * src.c2, r1 = ((Int)at[0][a] * src.c1 + at[1][1]) * src.c2;
+            const double x = mean(mean(MG5_AT(phic, r0 + at[2][0]), MG5_AT(phic, r0 + at[2][1])),
+                                  mean(MG5_AT(phic, r1 + at[2][0]), MG5_AT(phic, r1 + at[2][1])));
+            v = a == 0 ? x : mean(v, x);
+        }
+    }
+    MG5_AT(fine, t) = v;
 }
 
 static cudaError_t refine_any(const double *phic, const RefineSrc &src, const int o[3], int d0, int d1,
