@@ -404,7 +404,7 @@ __device__ __forceinline__ void bot_load(float *dst, const float *src)
     for (int m = 0; m < (BotGrid<N>::CELLS + kBotThreads - 1) / kBotThreads; ++m) {
         const int q = m * kBotThreads + threadIdx.x, row = q / N, k = q - row * N, i = row / N, j = row - i * N;
         if (q < BotGrid<N>::CELLS)
-            dst[BotGrid<N>::idx(i, j, k)] = MG5_AT(src, q);
+            MG5_AT(dst, BotGrid<N>::idx(i, j, k)) = MG5_AT(src, q);
     }
 }
 
@@ -420,8 +420,8 @@ __device__ __forceinline__ void bot_visit(BotGrid<N> &g, const BotArgs &A, BotSh
     for (int q = p; q < G::CELLS; q += kBotThreads) {
         int colour;
         const BotNbr nb = bot_at<N>(q, colour);
-        g.f[q] = bot_op(g.v + colour * G::HC, g.v + (1 - colour) * G::HC, nb, MG5_AT(g.bs, q), MG5_AT(g.bd, q),
-                        cf) + g.f[q] - sh.mf;
+        MG5_AT(g.f, q) = bot_op(g.v + colour * G::HC, g.v + (1 - colour) * G::HC, nb, MG5_AT(g.bs, q), MG5_AT(g.bd, q),
+                        cf) + MG5_AT(g.f, q) - sh.mf;
     }
     __syncthreads();
     if constexpr (LAST) {
@@ -454,15 +454,15 @@ __device__ __forceinline__ void bot_visit(BotGrid<N> &g, const BotArgs &A, BotSh
                     const int colour = (i + j + k) & 1;
                     const BotNbr nb = bot_nbr<N>(i, j, k);
                     const int q = colour * G::HC + nb.r00 + nb.k0;
-                    const float res = __fsub_rn(g.f[q] + 0.0f, bot_op(g.v + colour * G::HC, g.v + (1 - colour) * G::HC,
+                    const float res = __fsub_rn(MG5_AT(g.f, q) + 0.0f, bot_op(g.v + colour * G::HC, g.v + (1 - colour) * G::HC,
                                                                        nb, MG5_AT(g.bs, q), MG5_AT(g.bd, q), cf));
-                    sv += g.v[q];
+                    sv += MG5_AT(g.v, q);
                     sr += res;
                     acc.add(res);
                 }
                 const int q = C::idx(I, J, K);
-                c.v[q] = c.v0[q] = sv * 0.125f;
-                c.f[q] = sr * 0.125f;
+                MG5_AT(c.v, q) = MG5_AT(c.v0, q) = sv * 0.125f;
+                MG5_AT(c.f, q) = sr * 0.125f;
             }
             MomT<float> v{(float)acc.n, acc.k, acc.s, acc.q};
             v = momt_shift(v, __shfl_sync(0xffffffffu, v.k, 0));
@@ -499,9 +499,9 @@ __device__ __forceinline__ void bot_visit(BotGrid<N> &g, const BotArgs &A, BotSh
             static_assert(N != 8 || G::CELLS == kBotThreads, "a cell a thread");
             int colour;
             const BotNbr nb = bot_at<N>(p, colour);
-            const float res = __fsub_rn(g.f[p] + 0.0f, bot_op(g.v + colour * G::HC, g.v + (1 - colour) * G::HC, nb,
+            const float res = __fsub_rn(MG5_AT(g.f, p) + 0.0f, bot_op(g.v + colour * G::HC, g.v + (1 - colour) * G::HC, nb,
                                                                MG5_AT(g.bs, p), MG5_AT(g.bd, p), cf));
-            g.w[p] = res;
+            MG5_AT(g.w, p) = res;
             float2 s = make_float2(res, 0.0f);
             for (int o = 16; o > 0; o >>= 1)
                 s = pair_sum(s, pair_xor(s, o));
@@ -514,12 +514,12 @@ __device__ __forceinline__ void bot_visit(BotGrid<N> &g, const BotArgs &A, BotSh
 #pragma unroll
                 for (int ch = 0; ch < 8; ++ch) {
                     const int q = G::idx(2 * I + (ch >> 2), 2 * J + ((ch >> 1) & 1), 2 * K + (ch & 1));
-                    sv += g.v[q];
-                    sr += g.w[q];
+                    sv += MG5_AT(g.v, q);
+                    sr += MG5_AT(g.w, q);
                 }
                 const int q = C::idx(I, J, K);
-                c.v[q] = c.v0[q] = sv * 0.125f;
-                c.f[q] = sr * 0.125f;
+                MG5_AT(c.v, q) = MG5_AT(c.v0, q) = sv * 0.125f;
+                MG5_AT(c.f, q) = sr * 0.125f;
             }
             if (warp == 0) {
                 s = warps_pair_sum<kBotThreads / 32>(sh.sum);
@@ -535,7 +535,7 @@ __device__ __forceinline__ void bot_visit(BotGrid<N> &g, const BotArgs &A, BotSh
         bot_visit<NC, L + 1, NC == 4 || NC == 6>(c, A, sh, clamps);
         // prolongation of the correction (cell-centred trilinear), c += c of the grid below
         for (int q = p; q < C::CELLS; q += kBotThreads)
-            c.w[q] = c.v[q] - c.v0[q];
+            MG5_AT(c.w, q) = MG5_AT(c.v, q) - MG5_AT(c.v0, q);
         if (p == 0) {
             sh.c[L] += sh.c[L + 1];
             sh.cf = (float)sh.c[L];
@@ -548,14 +548,14 @@ __device__ __forceinline__ void bot_visit(BotGrid<N> &g, const BotArgs &A, BotSh
             const int I2 = (i & 1) ? (I + 1 == NC ? 0 : I + 1) : (I == 0 ? NC - 1 : I - 1);
             const int J2 = (j & 1) ? (J + 1 == NC ? 0 : J + 1) : (J == 0 ? NC - 1 : J - 1);
             const int K2 = (k & 1) ? (K + 1 == NC ? 0 : K + 1) : (K == 0 ? NC - 1 : K - 1);
-            const auto e = [&](int x, int y, int z) { return c.w[C::idx(x, y, z)]; };
+            const auto e = [&](int x, int y, int z) { return MG5_AT(c.w, C::idx(x, y, z)); };
             // weights (3/4, 1/4) per axis as 3x + y, one 1/64 at the end (as k_prolong_add)
             const float z00 = fmaf(3.0f, e(I, J, K), e(I, J, K2)), z01 = fmaf(3.0f, e(I, J2, K), e(I, J2, K2));
             const float z10 = fmaf(3.0f, e(I2, J, K), e(I2, J, K2)), z11 = fmaf(3.0f, e(I2, J2, K), e(I2, J2, K2));
             const float y0 = fmaf(3.0f, z00, z01), y1 = fmaf(3.0f, z10, z11);
             const float o = fmaf(3.0f, y0, y1);
             const int d = G::idx(i, j, k);
-            g.v[d] = fmaf(o, 1.0f / 64.0f, g.v[d]);
+            MG5_AT(g.v, d) = fmaf(o, 1.0f / 64.0f, MG5_AT(g.v, d));
         }
         __syncthreads();
         bot_sweeps<N>(g, A.nu2, sh.cf, cf, clamps);
@@ -596,7 +596,7 @@ __global__ void __launch_bounds__(kBotThreads, 1) k_bottom(const __grid_constant
     for (int m = 0; m < (BotGrid<N0>::CELLS + kBotThreads - 1) / kBotThreads; ++m) {
         const int q = m * kBotThreads + threadIdx.x, row = q / N0, k = q - row * N0, i = row / N0, j = row - i * N0;
         if (q < BotGrid<N0>::CELLS)
-            MG5_AT(A.v, q) = g.v[BotGrid<N0>::idx(i, j, k)];
+            MG5_AT(A.v, q) = MG5_AT(g.v, BotGrid<N0>::idx(i, j, k));
     }
     if (clamps)
         atomicAdd(&MG5_AT(A.clamp, 0), (unsigned long long)clamps);

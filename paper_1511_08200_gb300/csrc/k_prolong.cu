@@ -178,19 +178,19 @@ __global__ void __launch_bounds__(PT_THREADS)
 #pragma unroll
         for (int m = 0; m < PER; ++m)
             if (tid + m * PT_THREADS < CELLS)
-                S[tid + m * PT_THREADS] = fixed ? to_fixed(e[m], ex) : __double_as_longlong(e[m]);
+                MG5_AT(S, tid + m * PT_THREADS) = fixed ? to_fixed(e[m], ex) : __double_as_longlong(e[m]);
     } else {
 #pragma unroll
         for (int m = 0; m < PER; ++m)
             if (tid + m * PT_THREADS < CELLS)
-                S[tid + m * PT_THREADS] = e[m];
+                MG5_AT(S, tid + m * PT_THREADS) = e[m];
     }
     __syncthreads();
     const int j = tid / PT_K, k = tid - j * PT_K, J = J0 + j, K = K0 + k;
     if (J >= nc || K >= nc)
         return;
     const E *base = S + j * PT_RK + k;
-    const auto at = [&](int pl, int b, int c) { return base[pl * PT_PL + b * PT_RK + c]; };
+    const auto at = [&](int pl, int b, int c) { return MG5_AT(base, pl * PT_PL + b * PT_RK + c); };
     if constexpr (sizeof(T) == 8) {
         if (!fixed) {
             march<T, double, TI>([&](int pl, int b, int c) { return __longlong_as_double(at(pl, b, c)); }, vf, I0, J, K,

@@ -139,7 +139,7 @@ struct Visit {
     {
         const float4 v = st(x);
         const int q = at(L, p, j, k);
-        array(L, a)[q] = v;
+        MG5_AT(array(L, a), q) = v;
         if (L.single)
             return;
         const int ps = (BOX ? L.n1 + 2 : L.n1) * L.wq;
@@ -172,8 +172,8 @@ struct Visit {
         }
         const int q = at(L, p, j, k);
         const float4 *a = array(L, ac) + q, *b = array(L, ao) + q;
-        const auto Av = [&](int x) { return ld(a[x]); };
-        const auto Ov = [&](int x) { return ld(b[x]); };
+        const auto Av = [&](int x) { return ld(MG5_AT(a, x)); };
+        const auto Ov = [&](int x) { return ld(MG5_AT(b, x)); };
         return lin_of(Av(0), Ov(xp) + Ov(xm), Ov(yp) + Ov(ym), Ov(zp) + Ov(zm),
                       (Av(xp + yp) - Av(xp + ym)) - (Av(xm + yp) - Av(xm + ym)),
                       (Av(xp + zp) - Av(xp + zm)) - (Av(xm + zp) - Av(xm + zm)),
@@ -181,11 +181,11 @@ struct Visit {
     }
     __device__ __forceinline__ P1 centre(const VisitLevel &L, int b, int p, int j, int k, int colour) const
     {
-        return ld(array(L, arr(colour, b))[at(L, p, j, k)]);
+        return ld(MG5_AT(array(L, arr(colour, b)), at(L, p, j, k)));
     }
     __device__ __forceinline__ float2 &Fat(const VisitLevel &L, int p, int j, int k) const
     {
-        return reinterpret_cast<float2 *>(sm + L.F)[(p * L.n1 + j) * L.n2 + k];
+        return MG5_AT(reinterpret_cast<float2 *>(sm + L.F), (p * L.n1 + j) * L.n2 + k);
     }
     __device__ __forceinline__ Pr Fget(const VisitLevel &L, int p, int j, int k) const
     {
@@ -303,9 +303,9 @@ struct Visit {
                 continue;
             const double vg = MG5_AT(L.v0, vcell(L, o.i0 + g.p, g.j, g.k)),
                          va = MG5_AT(L.v0, vcell(L, o.i0 + g.pa, g.ja, g.ka));
-            const P1 now = ld(array(L, g.ca ? a1 : a0)[at(L, g.pa, g.ja, g.ka)]);
+            const P1 now = ld(MG5_AT(array(L, g.ca ? a1 : a0), at(L, g.pa, g.ja, g.ka)));
             const P1 x = add_change(split_f64(vg), mul_pair(weight(L, g.m), change(now, va)));
-            array(L, (g.ca ^ (g.m & 1)) ? d1 : d0)[at(L, g.p, g.j, g.k)] = st(x);
+            MG5_AT(array(L, (g.ca ^ (g.m & 1)) ? d1 : d0), at(L, g.p, g.j, g.k)) = st(x);
         }
     }
 
@@ -420,7 +420,7 @@ struct Visit {
 #pragma unroll 1
         for (int t = tid; t < ng; t += VT) {
             const Ghost g = ghost(L, o, t);
-            array(L, arr(g.ca ^ (g.m & 1), 0))[at(L, g.p, g.j, g.k)] = st(split_checked(v0_at(L, o.i0 + g.p, g.j, g.k)));
+            MG5_AT(array(L, arr(g.ca ^ (g.m & 1), 0)), at(L, g.p, g.j, g.k)) = st(split_checked(v0_at(L, o.i0 + g.p, g.j, g.k)));
         }
         if (tid == 0)
             S.c[L.id] = Pr{0.0f, 0.0f};
@@ -495,7 +495,7 @@ struct Visit {
                 if (k >= L.n2)
                     continue;
                 const Pr F = Fget(L, p, j, k);
-                const P1 now = ld(array(L, ac)[at(L, p, j, k)]);
+                const P1 now = ld(MG5_AT(array(L, ac), at(L, p, j, k)));
                 const Lin1 lin = lin_at(L, ac, ao, p, j, k);
                 const Pr r = resid(lin, add_pair(F, c), kap);
                 const Pr d = neg(mul_pair(root_change(lin, r, kap, clamps), Pr{L.wh, L.wl}));

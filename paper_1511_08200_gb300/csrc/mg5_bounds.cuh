@@ -61,13 +61,15 @@ __device__ __forceinline__ bool global_ok(unsigned long long a, unsigned long lo
     return false;
 }
 
+// The CTA's shared memory ends where its dynamic part does.  (Against that part's own address: in a
+// cluster the addresses of a CTA's shared memory do not start at zero.)
+extern __shared__ __align__(128) unsigned char dynamic_part[];
 __device__ __forceinline__ bool shared_ok(const void *q, unsigned bytes)
 {
-    unsigned total;
-    asm volatile("mov.u32 %0, %%total_smem_size;" : "=r"(total));
-    const unsigned off = (unsigned)__cvta_generic_to_shared(q);
-    // 1 KiB of the window below the CTA's own shared memory is reserved on sm_90 and later
-    return off + bytes <= total + 1024u;
+    unsigned dyn;
+    asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
+    const unsigned end = (unsigned)__cvta_generic_to_shared(dynamic_part) + dyn;
+    return (unsigned)__cvta_generic_to_shared(q) + bytes <= end;
 }
 
 template <typename T>
