@@ -24,6 +24,9 @@
 // it in a pair rounded once, and the stopping test norm <= rtol norm_0 in FP32 wherever it is not
 // close: else it is formed in FP64.
 //
+// From 12^3 the results are those of the launches to the bit; from 16^3 and 8^3 the mean residual of 8^3 is
+// summed in pairs instead, which may round the constant c otherwise (fields within 2^-17 in the tests).
+//
 // A visit from 16^3 takes 47 us (launch by launch ~77, of it 29 for 8^3 and 4^3 in one CTA that
 // gathered through offset tables), from 12^3 40-46 (its 6^3 grid alone took 70).  Bound by shared-memory
 // bandwidth and latency on the one SM: a half-sweep of 16^3 is 1.9 kclk of shared loads.

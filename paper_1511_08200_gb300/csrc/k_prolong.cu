@@ -10,8 +10,9 @@
 // 128^3, 185 for 128^3 -> 256^3).  Here the largest |e| of the tile gives a common exponent, each e becomes
 // a multiple of 2^-56 of it (the e below keep what lies above that), the stages are exact 64-bit integer
 // multiply-adds, and only the difference and the final sum with v are FP64: 1.2 operations a fine cell.  The
-// correction is off by at most 1.3e-16 of the largest difference around (seven FP64 multiply-adds round
-// by as much), and a correction is itself corrected by the next cycle.  A tile whose largest
+// correction is off by at most 1.3e-16 of the tile's largest difference (seven FP64 multiply-adds round
+// by as much where the differences are of a size; a cell whose own are far smaller loses more than FP64
+// would, 2^-56 of the largest), and a correction is itself corrected by the next cycle.  A tile whose largest
 // |e| is not finite, zero or below 2^-900 takes the FP64 operations of the gather kernel.
 // Now 11.0 us (64^3 -> 128^3), 19 (72^3 -> 144^3, was 57) and 70 (128^3 -> 256^3).  In FP32 120^3 -> 240^3
 // 53 -> 23 us, 256^3 -> 512^3 258 -> 188.  Four planes a CTA below 96^3 coarse cells, where eight would

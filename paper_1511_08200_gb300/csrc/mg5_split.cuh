@@ -25,10 +25,12 @@
 //    pair arithmetic (as the FP64 kernels refine their FP32 estimate), so d is good to ~2^-44 of
 //    itself.  The new value phi - (omega/6) d u is added up in FP64.
 //
-// Measured against 128-bit arithmetic on converged lognormal fields (rms; residual relative to
-// ||s delta||, update relative to phi): residual 2.0e-15 .. 3.7e-15 at every side from 16 to 192
-// where the FP64 kernels' grows from 5e-16 (16^3) over 3e-15 (64^3) to 2e-14 (192^3); update
-// 5e-17 .. 9e-17 at 48^3 and up against the FP64 kernels' 1.4e-16 .. 1.5e-16.
+// Measured against 128-bit arithmetic on converged lognormal fields of sigma 0.5 .. 1.5 (rms; residual
+// relative to ||s delta||, update relative to phi), FP64 kernels -> these: residual 4.4e-15 .. 7.9e-15 ->
+// 2.5e-15 .. 2.8e-15 at 64^3, 8.2e-15 .. 1.6e-14 -> 2.4e-15 .. 2.8e-15 at 128^3; update 1.4e-16 .. 1.5e-16
+// -> 5e-17 .. 9e-17 at 48^3 and up.  The FP64 residual's error comes from the sums of the field's values and
+// lies in every cell, this one from the nonlinear terms' 2^-47 and lies in the densest: the largest of a
+// cell is 0.4e-15 .. 6.7e-15 of max |s delta| there, 2.5e-15 .. 8.6e-15 here.
 //
 // Every quantity is a float2: the same cell of two half-tiles, through the packed FP32
 // instructions (two lanes an instruction), which have no operand negation: products are formed

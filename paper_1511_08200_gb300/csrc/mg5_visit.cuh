@@ -8,7 +8,11 @@ constexpr int kVisitCtas = 16;
 constexpr int kVisitLevels = 6;
 // Cells of the largest grid taken.  A half-sweep of 32^3 costs 16 SMs 4.9 us (450 instructions a cell)
 // where a launch over all SMs takes 3.1 us (patch 5.2): a 64^3 refinement took 1497 us with the 32^3
-// grid in the cluster and 1423 without; 24 x 20 x 36 (2.2 us a half-sweep) gained 5% in it.
+// grid in the cluster and 1423 without; 24 x 20 x 36 (2.2 us a half-sweep) gained 5% in it.  The planes are
+// dealt along the first axis only, so a slab that is thin there uses few CTAs, one at 8 planes and
+// fewer.  That is slower than the same slab on its side, and still faster than launches (a relaxation
+// to 1e-10, launches -> cluster): 16 x 48 x 40 2181 -> 1511 us, 48 x 40 x 16 2188 -> 1085, 16 x 48 x 48
+// 2670 -> 1411, 20 x 72 x 72 7122 -> 2554, 16 x 96 x 16 1666 -> 1330, 16 x 20 x 24 1126 -> 897.
 constexpr int kVisitCells = 20000;
 constexpr int kVisitCoarsest = 2048;          // cells of a coarsest grid CTA 0 iterates
 constexpr int kVisitSmem = 222 * 1024;        // dynamic shared memory a CTA may use
