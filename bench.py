@@ -834,8 +834,8 @@ def run_serving(mg, torch, dev, alpha, s, seconds, rate=200.0, slots=16, warm_s=
                 autotune=True, precision="mixed", max_backlog=1024):
     """Poisson arrivals at `rate` req/s for `seconds`: sides 16 round(10^U(log 32, log 256)/16),
     sigma ~ U(0.5, 2), tol 1e-6 or 1e-8 with p = 1/2, every request its own field (generated
-    ahead of its arrival on a side stream), all in one `precision` ("mixed": captured graphs
-    from the server's pool; "fp64": host-driven solves on the workers' contexts); admitted by
+    ahead of its arrival on a side stream), all in one `precision` (captured solves from the
+    server's pool); admitted by
     HBM footprint.  Latency = completion - arrival (server clock); the first `warm_s` seconds
     are discarded (a fifth of the run if that is shorter).  A server that falls behind (more
     than `max_backlog` requests submitted and not done) ends the run early: saturated."""
