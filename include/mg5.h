@@ -514,8 +514,8 @@ int mg5_step_resid_restrict_f32(mg5_ctx *ctx, const float *e, const float *f, co
  * grid above, m its mean r, B the base on grid N; p gives h (of grid N), alpha, nu1, nu2, nu_coarse and
  * omega.  e_out: the corrected e, c_out (host): the grid's compatibility constant.  e, f, B, e_out:
  * device, N^3 floats.  variant 0: one launch a step by the kernels that gather; 1: as the solves run it.
- * Both give the same values, to the bit where no grid of 8^3 lies below N or is it (its mean residual
- * is summed in another order).  Allocates and frees a hierarchy of N; synchronises the stream. */
+ * Both give the same values, to the bit where none of the grids is 8^3 or has a side that is a multiple
+ * of 32 (their mean residuals are summed in another order).  Allocates and frees a hierarchy of N; synchronises the stream. */
 int mg5_step_visit_f32(mg5_ctx *ctx, const float *e, const float *f, const float *B, double m, int N,
                        const mg5_params *p, int variant, float *e_out, double *c_out, void *stream);
 /* The same sweep by the fused kernel (one read and one write of phi per cell). */
